@@ -773,7 +773,7 @@ static int step_block_list(map_pool* pool, int G, const int** list) {
 }
 
 // launches of one step on buffer pool->cur; flips cur.  fused: also reduce alpha of the
-// new state into dyn (next dt) and the FP64 sums.
+// new state into dyn (next dt) and the FP64 sums (which the finalisation before it zeroed).
 static int step_launches(map_pool* pool, const map_params* p, bool fused) {
   const HostTree& t = pool->tree;
   StepLaunch S{};
@@ -825,9 +825,6 @@ static int step_launches(map_pool* pool, const map_params* p, bool fused) {
     return MAP_OK;
   };
   int rc;
-  if (fused) {
-    CK(cudaMemsetAsync(pool->sums, 0, sizeof(double) * kNV * pool->nprob, pool->stream));
-  }
   if (p->scheme == MAP_WENO) {
     rc = run(pool->buf[in], pool->buf[2], nullptr, 1, false);
     if (rc) return rc;
@@ -1074,7 +1071,9 @@ int map_step(map_pool* pool, const map_params* p) {
 static int advance_once(map_pool* pool, const map_params* p) {
   int rc = fill_on(pool, pool->cur);
   if (rc) return rc;
-  CK(launch_finalize(make_finalize(pool, p), pool->stream, &pool->launches));
+  FinalizeLaunch F = make_finalize(pool, p);
+  F.sums = pool->sums;
+  CK(launch_finalize(F, pool->stream, &pool->launches));
   return step_launches(pool, p, true);
 }
 

@@ -7,11 +7,22 @@ namespace mapgb {
 
 // dt, c_h, c_p and the psi damping factor of each problem from its alpha_g (Sec. 3.7
 // time step; Sec. 2 c_h and c_p; eq. MHD-5 damping exp(-dt c_h^2/c_p^2)).  Resets the
-// running alpha maximum for the next reduction.
-__global__ void finalize_kernel(FinalizeLaunch L) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= L.nprob) return;
-  ProbDyn d = L.dyn[p];
+// running alpha maximum for the next reduction and, for a fused step, zeroes the
+// conservation sums that the step accumulates.
+//
+// One problem per CTA of two warps.  The kernel is a chain of dependent FP64 operations (a
+// quotient, root, logarithm or exponential is 10-20 of them, each some 50 cycles on a pipe
+// of 1/64 of the FP32 rate), so its time is the longest chain: warp 0 takes dt and the three
+// dt/dx0 quotients, one per lane of a single division; warp 1 takes log(c_d) before dt is
+// known and then c_p and the damping.  (One thread per problem, everything in sequence, and a
+// memset of the sums beside it: 5.2 us more per step; 128^2 MMC, ten steps and state in and
+// out: 299 -> 247 us.)
+__global__ void __launch_bounds__(64) finalize_kernel(FinalizeLaunch L) {
+  const int p = blockIdx.x, lane = threadIdx.x & 31;
+  const bool dt_warp = threadIdx.x < 32;
+  const double log_cd = !dt_warp && L.cp_mode == MAP_CP_FROM_CD ? log(L.c_d) : 0.0;
+  const ProbDyn d = L.dyn[p];
+  __syncthreads();                       // both warps hold the maxima before they are reset
   const double ag = __longlong_as_double((long long)d.alpha_bits);
   double sig = ag;
   if (L.ch_mode == MAP_CH_FIXED && L.ch_fixed > sig) sig = L.ch_fixed;
@@ -31,20 +42,29 @@ __global__ void finalize_kernel(FinalizeLaunch L) {
   if (L.ch_mode == MAP_CH_AUTO) ch = ag;
   else if (L.ch_mode == MAP_CH_PAPER) ch = L.c_cfl * d.mindx / dt;
   else ch = L.ch_fixed;
-  const double cp = L.cp_mode == MAP_CP_FROM_CD ? sqrt(-dt * ch * ch / log(L.c_d)) : L.cp_fixed;
-  const double damp = cp > 0.0 ? exp(-dt * ch * ch / (cp * cp)) : 1.0;
-  d.dt = dt;
-  d.ch = ch;
-  d.cp = cp;
-  d.damp = damp;
-  d.alpha_g = ag;
-  d.alpha_bits = 0ull;
-  d.kmax_bits = 0ull;
-  d.dtc = dtc;
-  // per-dimension dt/dx at level 0; a level-L block takes 2^L of it, which is dt/dx_L
-  // exactly (dx_L = dx0 / 2^L as the host computes it), so blocks divide nothing
-  for (int k = 0; k < 3; ++k) d.lam0[k] = dt / d.dx0[k];
-  L.dyn[p] = d;
+  ProbDyn* o = L.dyn + p;
+  if (dt_warp) {
+    // per-dimension dt/dx at level 0; a level-L block takes 2^L of it, which is dt/dx_L
+    // exactly (dx_L = dx0 / 2^L as the host computes it), so blocks divide nothing
+    const double q = dt / (lane == 0 ? d.dx0[0] : lane == 1 ? d.dx0[1] : d.dx0[2]);
+    if (lane < 3) o->lam0[lane] = q;
+    if (lane == 0) {
+      o->dt = dt;
+      o->ch = ch;
+      o->alpha_g = ag;
+      o->dtc = dtc;
+      o->alpha_bits = 0ull;
+      o->kmax_bits = 0ull;
+    }
+  } else {
+    const double cp = L.cp_mode == MAP_CP_FROM_CD ? sqrt(-dt * ch * ch / log_cd) : L.cp_fixed;
+    const double damp = cp > 0.0 ? exp(-dt * ch * ch / (cp * cp)) : 1.0;
+    if (lane == 0) {
+      o->cp = cp;
+      o->damp = damp;
+    }
+    if (L.sums && lane < kNV) L.sums[(size_t)p * kNV + lane] = 0.0;
+  }
 }
 
 __global__ void zero_alpha_kernel(ProbDyn* dyn, int n) {
@@ -77,7 +97,7 @@ cudaError_t launch_speeds_out(const ProbDyn* dyn, int n, double* out, cudaStream
 
 cudaError_t launch_finalize(const FinalizeLaunch& L, cudaStream_t s, long long* cnt) {
   if (cnt) ++*cnt;
-  finalize_kernel<<<(L.nprob + 127) / 128, 128, 0, s>>>(L);
+  finalize_kernel<<<L.nprob, 64, 0, s>>>(L);
   return cudaGetLastError();
 }
 

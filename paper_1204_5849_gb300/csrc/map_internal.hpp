@@ -274,6 +274,7 @@ struct FinalizeLaunch {
   double c_cfl, eta, ch_fixed, cp_fixed, c_d, dt_override;
   int ch_mode, cp_mode;
   int conduction = 0, subcycle = 1;   // conduction on: dt_c; without the subcycle dt <= dt_c
+  double* sums = nullptr;  // optional: conservation sums [nprob][9] to zero for the fused step after it
 };
 
 struct FlagLaunch {
