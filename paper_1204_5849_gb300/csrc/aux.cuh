@@ -1,6 +1,7 @@
 // aux.cuh -- ghost fill, restriction, CFL reduction, refinement flags, conservation sums,
 // host-layout packing and regrid kernels.
 #pragma once
+#include "chain.cuh"
 #include "map_internal.hpp"
 #include "physics.cuh"
 #include "step.cuh"
@@ -56,6 +57,7 @@ __global__ void __launch_bounds__(256) fill_kernel(T* __restrict__ u, const int*
   using SH = Shell<NDIM, NB>;
   constexpr int NP = G::NP, P2 = G::P2, S = G::S;
   __shared__ GhostRegion reg[27];
+  chain_begin();
   for (int bi = blockIdx.x; bi < n; bi += gridDim.x) {
     const int blk = blocks[bi];
     __syncthreads();
@@ -114,6 +116,7 @@ __global__ void __launch_bounds__(256) restrict_kernel(T* __restrict__ u, const 
   using G = Geo<NDIM, NB>;
   constexpr int NP = G::NP, P2 = G::P2, S = G::S;
   constexpr int NI = NDIM == 3 ? NB * NB * NB : NB * NB;
+  chain_begin();
   for (int bi = blockIdx.x; bi < n; bi += gridDim.x) {
     const int par = parents[bi];
     int ch[8];
@@ -167,6 +170,7 @@ __global__ void __launch_bounds__(256) cfl_kernel(const T* __restrict__ u, const
   P.gm1 = gm1;
   P.ch = T(0);
   P.tau = T(0);
+  chain_begin();
   for (int bi = blockIdx.x; bi < n; bi += gridDim.x) {
     const int blk = blocks[bi];
     const T* ub = u + (size_t)blk * NV * S;
@@ -462,6 +466,7 @@ __global__ void __launch_bounds__(256) reflux_kernel(RefluxLaunch L) {
   constexpr size_t NB2 = (size_t)NB * NB;
   constexpr size_t PER = (size_t)2 * NDIM * NV * NB2;   // one register slot
   __shared__ double red[NV + 1][32];
+  chain_begin();
   const RefluxTask& tk = L.tasks[blockIdx.x];
   const int q = tk.coarse;
   const BlockGeo gg = L.geo[q];
@@ -693,6 +698,7 @@ __global__ void __launch_bounds__(256) conduction_kernel(CondLaunch L) {
   extern __shared__ __align__(16) unsigned char csm[];
   T* sT = reinterpret_cast<T*>(csm);
   T* sK = sT + NR;
+  chain_begin();
   const int blk = L.blocks[blockIdx.x];
   const BlockGeo gg = L.geo[blk];
   if (L.it >= L.nsub[gg.problem]) return;

@@ -1,6 +1,7 @@
 // common.cu -- per-problem time-step finalisation (precision independent).
 #include <math.h>
 
+#include "chain.cuh"
 #include "map_internal.hpp"
 
 namespace mapgb {
@@ -21,6 +22,7 @@ __global__ void __launch_bounds__(64) finalize_kernel(FinalizeLaunch L) {
   const int p = blockIdx.x, lane = threadIdx.x & 31;
   const bool dt_warp = threadIdx.x < 32;
   const double log_cd = !dt_warp && L.cp_mode == MAP_CP_FROM_CD ? log(L.c_d) : 0.0;
+  chain_begin();
   const ProbDyn d = L.dyn[p];
   __syncthreads();                       // both warps hold the maxima before they are reset
   const double ag = __longlong_as_double((long long)d.alpha_bits);
@@ -68,6 +70,7 @@ __global__ void __launch_bounds__(64) finalize_kernel(FinalizeLaunch L) {
 }
 
 __global__ void zero_alpha_kernel(ProbDyn* dyn, int n) {
+  chain_begin();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n) {
     dyn[p].alpha_bits = 0ull;
@@ -97,14 +100,12 @@ cudaError_t launch_speeds_out(const ProbDyn* dyn, int n, double* out, cudaStream
 
 cudaError_t launch_finalize(const FinalizeLaunch& L, cudaStream_t s, long long* cnt) {
   if (cnt) ++*cnt;
-  finalize_kernel<<<L.nprob, 64, 0, s>>>(L);
-  return cudaGetLastError();
+  return launch_chained(finalize_kernel, L.nprob, 64, 0, s, L);
 }
 
 cudaError_t launch_zero_alpha(ProbDyn* dyn, int n, cudaStream_t s, long long* cnt) {
   if (cnt) ++*cnt;
-  zero_alpha_kernel<<<(n + 127) / 128, 128, 0, s>>>(dyn, n);
-  return cudaGetLastError();
+  return launch_chained(zero_alpha_kernel, (n + 127) / 128, 128, 0, s, dyn, n);
 }
 
 }  // namespace mapgb

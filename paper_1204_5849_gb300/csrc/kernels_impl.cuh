@@ -2,6 +2,7 @@
 // Included once per precision by kernels_f64.cu and kernels_f32.cu.
 #pragma once
 #include "aux.cuh"
+#include "chain.cuh"
 #include "step.cuh"
 
 namespace mapgb {
@@ -43,8 +44,7 @@ cudaError_t launch_step_one(const StepLaunch& L, cudaStream_t s) {
   A.fail_waits = L.fail_waits;
   const int grid = L.grid > 0 ? (L.grid < L.nblocks ? L.grid : L.nblocks) : L.nblocks;
   if (grid <= 0) return cudaSuccess;
-  kern<<<grid, step_threads<T, NDIM, NB>(), smem, s>>>(A);
-  return cudaGetLastError();
+  return launch_chained(kern, grid, step_threads<T, NDIM, NB>(), smem, s, A);
 }
 
 // Each (FLX, RFX) pair is instantiated in its own translation unit (kernels_<prec>.cu,
@@ -115,9 +115,8 @@ cudaError_t launch_fill_T(const KernelConfig& kc, const FillLaunch& L, cudaStrea
   if (L.nblocks <= 0) return cudaSuccess;
   if (cnt) ++*cnt;
 #define CALL_FILL(ND, NBV)                                                                   \
-  fill_kernel<T, ND, NBV><<<grid_for(L.nblocks), 256, 0, s>>>((T*)L.u, L.blocks, L.nblocks, L.regions, L.skip_pushed, \
-                                                              L.v0, L.v1);                                \
-  return cudaGetLastError()
+  return launch_chained(fill_kernel<T, ND, NBV>, grid_for(L.nblocks), 256, 0, s, (T*)L.u, L.blocks, L.nblocks, \
+                        L.regions, L.skip_pushed, L.v0, L.v1)
   MAPGB_GEO_DISPATCH(kc, CALL_FILL);
 #undef CALL_FILL
 }
@@ -127,8 +126,8 @@ cudaError_t launch_restrict_T(const KernelConfig& kc, const RestrictLaunch& L, c
   if (L.nparents <= 0) return cudaSuccess;
   if (cnt) ++*cnt;
 #define CALL_RES(ND, NBV)                                                                          \
-  restrict_kernel<T, ND, NBV><<<grid_for(L.nparents), 256, 0, s>>>((T*)L.u, L.parents, L.nparents, L.children); \
-  return cudaGetLastError()
+  return launch_chained(restrict_kernel<T, ND, NBV>, grid_for(L.nparents), 256, 0, s, (T*)L.u, L.parents, L.nparents, \
+                        L.children)
   MAPGB_GEO_DISPATCH(kc, CALL_RES);
 #undef CALL_RES
 }
@@ -138,9 +137,8 @@ cudaError_t launch_cfl_T(const KernelConfig& kc, const CflLaunch& L, cudaStream_
   if (L.nblocks <= 0) return cudaSuccess;
   if (cnt) ++*cnt;
 #define CALL_CFL(ND, NBV)                                                                     \
-  cfl_kernel<T, ND, NBV><<<grid_for(L.nblocks), 256, 0, s>>>((const T*)L.u, L.blocks, L.nblocks, L.geo, L.dyn, \
-                                                             (T)L.gamma, (T)(L.gamma - 1.0), L.kappa0); \
-  return cudaGetLastError()
+  return launch_chained(cfl_kernel<T, ND, NBV>, grid_for(L.nblocks), 256, 0, s, (const T*)L.u, L.blocks, L.nblocks, \
+                        L.geo, L.dyn, (T)L.gamma, (T)(L.gamma - 1.0), L.kappa0)
   MAPGB_GEO_DISPATCH(kc, CALL_CFL);
 #undef CALL_CFL
 }
@@ -194,8 +192,7 @@ cudaError_t launch_reflux_T(const KernelConfig& kc, const RefluxLaunch& L, cudaS
   if (L.ntasks <= 0) return cudaSuccess;
   if (cnt) ++*cnt;
 #define CALL_REFLUX(ND, NBV)                                              \
-  reflux_kernel<T, ND, NBV><<<L.ntasks, 256, 0, s>>>(L);                  \
-  return cudaGetLastError()
+  return launch_chained(reflux_kernel<T, ND, NBV>, L.ntasks, 256, 0, s, L)
   MAPGB_GEO_DISPATCH(kc, CALL_REFLUX);
 #undef CALL_REFLUX
 }
@@ -211,8 +208,7 @@ cudaError_t launch_conduction_one(const CondLaunch& L, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     attr_done = true;
   }
-  kern<<<L.nblocks, 256, smem, s>>>(L);
-  return cudaGetLastError();
+  return launch_chained(kern, L.nblocks, 256, smem, s, L);
 }
 
 template <typename T>

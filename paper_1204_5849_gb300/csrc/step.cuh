@@ -24,6 +24,7 @@
 #pragma once
 #include <type_traits>
 
+#include "chain.cuh"
 #include "map_internal.hpp"
 #include "physics.cuh"
 
@@ -506,6 +507,7 @@ step_kernel(StepArgsT<T> A) {
       for (int k = 0; k < 16; ++k) sched[q][k] = A.sched[q][k];
   }
   __syncthreads();
+  chain_begin();
   unsigned phase = 0;                                   // parity bit per u slot
   unsigned inflight = 0;                                // thread 0: slots with copies in flight
 
