@@ -165,13 +165,32 @@ cudaError_t launch_sums_T(const KernelConfig& kc, const SumLaunch& L, cudaStream
 #undef CALL_SUMS
 }
 
+template <typename T, typename H, int NDIM, int NB, int W>
+cudaError_t launch_pack_one(const PackLaunch& L, cudaStream_t s) {
+  constexpr long long per = (long long)NV * (NDIM == 3 ? NB * NB * NB : NB * NB) / W;
+  const long long ctas = (L.nblocks * per + PackShape::PER_CTA - 1) / PackShape::PER_CTA;
+  H* dense = reinterpret_cast<H*>(L.host_layout);
+  if (L.to_pool)
+    pack_kernel<T, H, NDIM, NB, W, true><<<(unsigned)ctas, PackShape::THREADS, 0, s>>>((T*)L.u, dense, L.blocks, L.nblocks);
+  else
+    pack_kernel<T, H, NDIM, NB, W, false><<<(unsigned)ctas, PackShape::THREADS, 0, s>>>((T*)L.u, dense, L.blocks, L.nblocks);
+  return cudaGetLastError();
+}
+
+template <typename T, int NDIM, int NB>
+cudaError_t launch_pack_geo(const PackLaunch& L, cudaStream_t s) {
+  const size_t elem = L.staging_f32 ? sizeof(float) : sizeof(double);
+  const bool wide = (uintptr_t)L.host_layout % (4 * elem) == 0;   // the library's own staging always is
+  if (L.staging_f32)
+    return wide ? launch_pack_one<T, float, NDIM, NB, 4>(L, s) : launch_pack_one<T, float, NDIM, NB, 1>(L, s);
+  return wide ? launch_pack_one<T, double, NDIM, NB, 4>(L, s) : launch_pack_one<T, double, NDIM, NB, 1>(L, s);
+}
+
 template <typename T>
 cudaError_t launch_pack_T(const KernelConfig& kc, const PackLaunch& L, cudaStream_t s, long long* cnt) {
   if (L.nblocks <= 0) return cudaSuccess;
   if (cnt) ++*cnt;
-#define CALL_PACK(ND, NBV)                                             \
-  pack_kernel<T, ND, NBV><<<grid_for(L.nblocks), 256, 0, s>>>(L);      \
-  return cudaGetLastError()
+#define CALL_PACK(ND, NBV) return launch_pack_geo<T, ND, NBV>(L, s)
   MAPGB_GEO_DISPATCH(kc, CALL_PACK);
 #undef CALL_PACK
 }
