@@ -8,103 +8,127 @@
 
 namespace mapgb {
 
+// W neighbouring values moved by one access
+template <typename T, int W>
+struct alignas(W * sizeof(T)) Pack {
+  T v[W];
+};
+
 // Ghost fill of the leaves of one level (Sec. 4.3): every ghost cell gathers from the
 // block its region resolves to -- a copy from a same-level block, or the conservative
 // minmod prolongation of the covering coarser leaf (whose ghosts an earlier level pass
 // filled).  Region tables come from the host tree.
+//
+// A thread takes a pair of x-neighbours (2p, 2p + 1) of one leaf, all variables: the two
+// ghost columns of a side, like every pair inside the block's x range, lie in one region, and
+// every unclamped index map shifts x by an even number, so a copied pair is one 8-byte (FP32)
+// load and store per variable and a prolonged pair has one coarse cell, whose slopes it
+// shares.  Pairs are numbered over all leaves, so small blocks leave no threads idle.
+// Latency- and instruction-bound before (one cell per thread, one CTA per leaf); a fill of
+// every region: 256^3 FP32 456 us -> 402, octree of 9472 8^3 leaves, finest level 222 ->
+// 191, 32640 16^2 blocks 181 -> 154.
 template <int NDIM, int NB>
 struct Shell {
   static constexpr int NP = NB + 4;
-  static constexpr int P2 = NP * NP;
-  static constexpr int PLANE_GHOSTS = P2 - NB * NB;                  // ghost cells of an interior plane
-  static constexpr int COUNT = NDIM == 3 ? 2 * NG * P2 + NB * PLANE_GHOSTS : PLANE_GHOSTS;
-  // g-th ghost cell of a block -> padded (i, j, k): the 2*NG full ghost planes first (3D),
-  // then per interior plane its NG ghost rows on each side and NG ghost columns on each side
-  static __device__ __forceinline__ void cell(int g, int& i, int& j, int& k) {
+  static constexpr int ROW = NP / 2;                                 // pairs of a padded row
+  static constexpr int PLANE = NP * ROW;
+  static constexpr int PLANE_GHOSTS = 2 * NG * ROW + NB * NG;        // pairs: ghost rows, then ghost columns
+  static constexpr int COUNT = NDIM == 3 ? 2 * NG * PLANE + NB * PLANE_GHOSTS : PLANE_GHOSTS;
+  // g-th ghost pair of a block -> padded (i, j, k) of its first cell: the 2*NG full ghost
+  // planes first (3D), then per interior plane its NG ghost rows on each side and the pair of
+  // ghost columns on each side
+  static __device__ __forceinline__ void pair(int g, int& i, int& j, int& k) {
     if (NDIM == 3) {
-      if (g < 2 * NG * P2) {
-        const int pl = g / P2, c = g % P2;
+      if (g < 2 * NG * PLANE) {
+        const int pl = g / PLANE, c = g % PLANE;
         k = pl < NG ? pl : NB + pl;
-        j = c / NP;
-        i = c % NP;
+        j = c / ROW;
+        i = 2 * (c % ROW);
         return;
       }
-      g -= 2 * NG * P2;
+      g -= 2 * NG * PLANE;
       k = NG + g / PLANE_GHOSTS;
       g %= PLANE_GHOSTS;
     } else {
       k = 0;
     }
-    constexpr int ROWS = 2 * NG * NP;          // full ghost rows of the plane
+    constexpr int ROWS = 2 * NG * ROW;
     if (g < ROWS) {
-      const int r = g / NP;
+      const int r = g / ROW;
       j = r < NG ? r : NB + r;
-      i = g % NP;
+      i = 2 * (g % ROW);
     } else {
-      g -= ROWS;                                // NB interior rows x 2*NG ghost columns
-      j = NG + g / (2 * NG);
-      const int q = g % (2 * NG);
-      i = q < NG ? q : NB + q;
+      g -= ROWS;
+      j = NG + g / 2;
+      i = g % 2 ? NB + NG : 0;
     }
   }
 };
 
-template <typename T, int NDIM, int NB>
+// EONLY: the energy alone (between conduction substeps)
+template <typename T, int NDIM, int NB, bool EONLY>
 __global__ void __launch_bounds__(256) fill_kernel(T* __restrict__ u, const int* __restrict__ blocks,
-                                                   int n, const GhostRegion* __restrict__ regions, int skip_pushed,
-                                                   int v0, int v1) {
+                                                   int n, const GhostRegion* __restrict__ regions, int skip_pushed) {
   using G = Geo<NDIM, NB>;
   using SH = Shell<NDIM, NB>;
+  using P = Pack<T, 2>;
   constexpr int NP = G::NP, P2 = G::P2, S = G::S;
-  __shared__ GhostRegion reg[27];
+  constexpr int V0 = EONLY ? EN : 0, V1 = EONLY ? EN + 1 : NV;
+  static_assert(NG == 2 && NP % 2 == 0, "the ghost columns of a side are one aligned pair");
   chain_begin();
-  for (int bi = blockIdx.x; bi < n; bi += gridDim.x) {
-    const int blk = blocks[bi];
-    __syncthreads();
-    for (int r = threadIdx.x; r < 27; r += blockDim.x) reg[r] = regions[(size_t)blk * 27 + r];
-    __syncthreads();
-    T* ub = u + (size_t)blk * NV * S;
-    for (int g = threadIdx.x; g < SH::COUNT; g += blockDim.x) {
-      int i, j, k;
-      SH::cell(g, i, j, k);
-      const int c = (k * NP + j) * NP + i;
-      const int rx = i < NG ? 0 : (i >= NG + NB ? 2 : 1);
-      const int ry = j < NG ? 0 : (j >= NG + NB ? 2 : 1);
-      const int rz = NDIM == 3 ? (k < NG ? 0 : (k >= NG + NB ? 2 : 1)) : 1;
-      const GhostRegion& gr = reg[rx + 3 * ry + 9 * rz];
-      if (skip_pushed && gr.pushed) continue;      // written by the source's step kernel
-      const T* sb = u + (size_t)gr.src * NV * S;
-      if (gr.kind == 0) {
-        const int si = gr.m[0] * i + gr.a[0], sj = gr.m[1] * j + gr.a[1];
-        const int sk = NDIM == 3 ? gr.m[2] * k + gr.a[2] : 0;
-        const int sc = (sk * NP + sj) * NP + si;
-        T val[NV];
+  // (32-bit: a pool that fills the device's memory has under 2^30 ghost pairs)
+  const unsigned item = blockIdx.x * blockDim.x + threadIdx.x;
+  const int leaf = (int)(item / SH::COUNT), g = (int)(item % SH::COUNT);
+  if (leaf >= n) return;
+  const int blk = blocks[leaf];
+  int i, j, k;
+  SH::pair(g, i, j, k);
+  const int c = (k * NP + j) * NP + i;
+  const int rx = i < NG ? 0 : (i >= NG + NB ? 2 : 1);
+  const int ry = j < NG ? 0 : (j >= NG + NB ? 2 : 1);
+  const int rz = NDIM == 3 ? (k < NG ? 0 : (k >= NG + NB ? 2 : 1)) : 1;
+  const GhostRegion gr = regions[(size_t)blk * 27 + rx + 3 * ry + 9 * rz];
+  if (skip_pushed && gr.pushed) return;            // written by the source's step kernel
+  T* ub = u + (size_t)blk * NV * S + c;
+  const T* sb = u + (size_t)gr.src * NV * S;
+  const int gi = gr.m[0] * i + gr.a[0], gj = gr.m[1] * j + gr.a[1];
+  const int gk = NDIM == 3 ? gr.m[2] * k + gr.a[2] : 0;
+  const bool mapped = gr.m[0] == 1;                // else both cells clamp to one x index
+  if (gr.kind == 0) {
+    const T* f = sb + (gk * NP + gj) * NP + gi;
+    P val[NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v)
-          if (v >= v0 && v < v1) val[v] = sb[(size_t)v * S + sc];
+    for (int v = V0; v < V1; ++v) {
+      if (mapped) val[v] = *reinterpret_cast<const P*>(f + (size_t)v * S);
+      else val[v].v[0] = val[v].v[1] = f[(size_t)v * S];
+    }
 #pragma unroll
-        for (int v = 0; v < NV; ++v)
-          if (v >= v0 && v < v1) ub[(size_t)v * S + c] = val[v];
-      } else {
-        const int gi = gr.m[0] * i + gr.a[0], gj = gr.m[1] * j + gr.a[1];
-        const int gk = NDIM == 3 ? gr.m[2] * k + gr.a[2] : 0;
-        const int ci = (gi >> 1) - gr.corg[0] + NG, cj = (gj >> 1) - gr.corg[1] + NG;
-        const int ck = NDIM == 3 ? (gk >> 1) - gr.corg[2] + NG : 0;
-        const int cc = (ck * NP + cj) * NP + ci;
-        const T ox = (gi & 1) ? T(0.25) : T(-0.25);
-        const T oy = (gj & 1) ? T(0.25) : T(-0.25);
-        const T oz = (gk & 1) ? T(0.25) : T(-0.25);
+    for (int v = V0; v < V1; ++v) *reinterpret_cast<P*>(ub + (size_t)v * S) = val[v];
+  } else {
+    const int ci = (gi >> 1) - gr.corg[0] + NG, cj = (gj >> 1) - gr.corg[1] + NG;
+    const int ck = NDIM == 3 ? (gk >> 1) - gr.corg[2] + NG : 0;
+    const T* fc = sb + (ck * NP + cj) * NP + ci;
+    // mapped: gi is even, so the pair covers both halves of coarse cell ci
+    const T ox0 = (gi & 1) ? T(0.25) : T(-0.25), ox1 = mapped ? T(0.25) : ox0;
+    const T oy = (gj & 1) ? T(0.25) : T(-0.25);
+    const T oz = (gk & 1) ? T(0.25) : T(-0.25);
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          if (v < v0 || v >= v1) continue;
-          const T* f = sb + (size_t)v * S;
-          T val = f[cc];
-          val += minmod<T>(f[cc + 1] - f[cc], f[cc] - f[cc - 1]) * ox;
-          val += minmod<T>(f[cc + NP] - f[cc], f[cc] - f[cc - NP]) * oy;
-          if (NDIM == 3) val += minmod<T>(f[cc + P2] - f[cc], f[cc] - f[cc - P2]) * oz;
-          ub[(size_t)v * S + c] = val;
-        }
+    for (int v = V0; v < V1; ++v) {
+      const T* f = fc + (size_t)v * S;
+      const T f0 = f[0];
+      const T sx = minmod<T>(f[1] - f0, f0 - f[-1]);
+      const T sy = minmod<T>(f[NP] - f0, f0 - f[-NP]);
+      const T sz = NDIM == 3 ? minmod<T>(f[P2] - f0, f0 - f[-P2]) : T(0);
+      P val;
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        T t = f0;
+        t += sx * (x ? ox1 : ox0);
+        t += sy * oy;
+        if (NDIM == 3) t += sz * oz;
+        val.v[x] = t;
       }
+      *reinterpret_cast<P*>(ub + (size_t)v * S) = val;
     }
   }
 }
@@ -391,11 +415,6 @@ __global__ void __launch_bounds__(256) sums_kernel(SumLaunch L) {
 // same walk with single values, for a caller's buffer that is not aligned to four of them.
 // 256^3 FP32 to the pool and back: 343 + 445 us one value per access -> 197 + 320 (floor 178
 // each at the copy rate).
-template <typename T, int W>
-struct alignas(W * sizeof(T)) Pack {
-  T v[W];
-};
-
 struct PackShape {
   static constexpr int THREADS = 192, QUADS = 3, PER_CTA = THREADS * QUADS;
 };

@@ -589,8 +589,7 @@ static int fill_energy_on(map_pool* pool, int q) {
     F.nblocks = D.leaf_off[L + 1] - D.leaf_off[L];
     F.regions = D.regions;
     F.skip_pushed = 0;
-    F.v0 = kEN;
-    F.v1 = kEN + 1;
+    F.energy_only = 1;
     CK(DISPATCH(pool, fill, F));
   }
   return MAP_OK;

@@ -115,8 +115,9 @@ cudaError_t launch_fill_T(const KernelConfig& kc, const FillLaunch& L, cudaStrea
   if (L.nblocks <= 0) return cudaSuccess;
   if (cnt) ++*cnt;
 #define CALL_FILL(ND, NBV)                                                                   \
-  return launch_chained(fill_kernel<T, ND, NBV>, grid_for(L.nblocks), 256, 0, s, (T*)L.u, L.blocks, L.nblocks, \
-                        L.regions, L.skip_pushed, L.v0, L.v1)
+  return launch_chained(L.energy_only ? fill_kernel<T, ND, NBV, true> : fill_kernel<T, ND, NBV, false>, \
+                        (int)(((long long)L.nblocks * Shell<ND, NBV>::COUNT + 255) / 256), 256, 0, s, (T*)L.u, \
+                        L.blocks, L.nblocks, L.regions, L.skip_pushed)
   MAPGB_GEO_DISPATCH(kc, CALL_FILL);
 #undef CALL_FILL
 }

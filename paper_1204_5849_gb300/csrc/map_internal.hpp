@@ -40,7 +40,7 @@ struct ProbDyn {
 //   kind 0 COPY:    src block interior/any cell at padded index (m*i + a)
 //   kind 1 PROLONG: fine global cell g = m*i + a; coarse padded = (g >> 1) - corg + NG,
 //                   offset sign from g & 1 (minmod-linear, Sec. 4.3)
-struct GhostRegion {
+struct alignas(16) GhostRegion {   // 48 bytes: three 16-byte loads
   int kind;
   int src;
   int m[3];
@@ -247,7 +247,7 @@ struct FillLaunch {
   int nblocks;
   const GhostRegion* regions;
   int skip_pushed;         // 1: leave regions the previous step kernel wrote
-  int v0 = 0, v1 = kNV;    // variables filled: [v0, v1)
+  int energy_only = 0;     // 1: the energy alone
 };
 
 struct RestrictLaunch {
