@@ -133,37 +133,57 @@ __global__ void __launch_bounds__(256) fill_kernel(T* __restrict__ u, const int*
   }
 }
 
-// Parents of one level become the mean of their 2^ndim children (Sec. 4.3 step (1)).
+// Parents of one level become the mean of their 2^ndim children (Sec. 4.3 step (1)).  A thread
+// takes one variable of ITEMS parent cells, and a parent is spread over several CTAs (its
+// cells and variables are a whole number of CTAs): levels hold few parents.  The two
+// x-children of a cell are one aligned pair.  One CTA per parent with the variables in
+// sequence was bound by their load latencies: 2D 16^2, 680, 232 and 64 parents: 10, 8
+// and 8 us -> 9.5, 5.4 and 4.7 (cold caches; a quadtree step does six); 1088 8^3 parents 60 -> 54.
+struct RestrictShape {
+  static constexpr int THREADS = 192, ITEMS = 3, PER_CTA = THREADS * ITEMS;
+};
+
 template <typename T, int NDIM, int NB>
-__global__ void __launch_bounds__(256) restrict_kernel(T* __restrict__ u, const int* __restrict__ parents,
-                                                       int n, const int* __restrict__ children) {
+__global__ void __launch_bounds__(RestrictShape::THREADS) restrict_kernel(T* __restrict__ u, const int* __restrict__ parents,
+                                                                              const int* __restrict__ children) {
   using G = Geo<NDIM, NB>;
-  constexpr int NP = G::NP, P2 = G::P2, S = G::S;
+  using P = Pack<T, 2>;
+  constexpr int NP = G::NP, S = G::S;
   constexpr int NI = NDIM == 3 ? NB * NB * NB : NB * NB;
+  constexpr int NZC = NDIM == 3 ? 2 : 1;
+  constexpr int N = RestrictShape::ITEMS, M = NV * NI / RestrictShape::PER_CTA;   // CTAs per parent
+  static_assert(NV * NI % RestrictShape::PER_CTA == 0, "a parent is a whole number of CTAs");
   chain_begin();
-  for (int bi = blockIdx.x; bi < n; bi += gridDim.x) {
-    const int par = parents[bi];
-    int ch[8];
+  const int par = parents[blockIdx.x / M];
+  T* dst[N];
+  P f[N][NZC][2];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) ch[q] = children[(size_t)par * 8 + q];
-    T* pb = u + (size_t)par * NV * S;
-    for (int c = threadIdx.x; c < NI; c += blockDim.x) {
-      const int i = c % NB, j = (c / NB) % NB, k = NDIM == 3 ? c / (NB * NB) : 0;
-      const int dst = ((NDIM == 3 ? k + NG : 0) * NP + j + NG) * NP + i + NG;
-#pragma unroll 1
-      for (int v = 0; v < NV; ++v) {
-        T sum = T(0);
-        for (int dz = 0; dz < (NDIM == 3 ? 2 : 1); ++dz)
-          for (int dy = 0; dy < 2; ++dy)
-            for (int dx = 0; dx < 2; ++dx) {
-              const int fi = 2 * i + dx, fj = 2 * j + dy, fk = 2 * k + dz;
-              const int cb = (fi / NB) | ((fj / NB) << 1) | ((NDIM == 3 ? fk / NB : 0) << 2);
-              const int lc = ((NDIM == 3 ? fk % NB + NG : 0) * NP + fj % NB + NG) * NP + fi % NB + NG;
-              sum += u[(size_t)ch[cb] * NV * S + (size_t)v * S + lc];
-            }
-        pb[(size_t)v * S + dst] = sum / T(1 << NDIM);
+  for (int q = 0; q < N; ++q) {
+    const int r = (blockIdx.x % M) * RestrictShape::PER_CTA + q * RestrictShape::THREADS + threadIdx.x;
+    const int v = r / NI, c = r % NI;
+    const int i = c % NB, j = (c / NB) % NB, k = NDIM == 3 ? c / (NB * NB) : 0;
+    const int fi = 2 * i, fj = 2 * j, fk = 2 * k;
+    // both halves of a cell's children lie in one child block (NB is even)
+    const int cb = (fi / NB) | ((fj / NB) << 1) | ((NDIM == 3 ? fk / NB : 0) << 2);
+    const T* src = u + (size_t)children[(size_t)par * 8 + cb] * NV * S + (size_t)v * S +
+                   ((NDIM == 3 ? fk % NB + NG : 0) * NP + fj % NB + NG) * NP + fi % NB + NG;
+    dst[q] = u + (size_t)par * NV * S + (size_t)v * S + ((NDIM == 3 ? k + NG : 0) * NP + j + NG) * NP + i + NG;
+#pragma unroll
+    for (int dz = 0; dz < NZC; ++dz)
+#pragma unroll
+      for (int dy = 0; dy < 2; ++dy) f[q][dz][dy] = *reinterpret_cast<const P*>(src + (dz * NP + dy) * NP);
+  }
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    T sum = T(0);
+#pragma unroll
+    for (int dz = 0; dz < NZC; ++dz)
+#pragma unroll
+      for (int dy = 0; dy < 2; ++dy) {
+        sum += f[q][dz][dy].v[0];
+        sum += f[q][dz][dy].v[1];
       }
-    }
+    *dst[q] = sum / T(1 << NDIM);
   }
 }
 

@@ -127,8 +127,9 @@ cudaError_t launch_restrict_T(const KernelConfig& kc, const RestrictLaunch& L, c
   if (L.nparents <= 0) return cudaSuccess;
   if (cnt) ++*cnt;
 #define CALL_RES(ND, NBV)                                                                          \
-  return launch_chained(restrict_kernel<T, ND, NBV>, grid_for(L.nparents), 256, 0, s, (T*)L.u, L.parents, L.nparents, \
-                        L.children)
+  return launch_chained(restrict_kernel<T, ND, NBV>, \
+                        L.nparents * (NV * (ND == 3 ? NBV * NBV * NBV : NBV * NBV) / RestrictShape::PER_CTA), \
+                        RestrictShape::THREADS, 0, s, (T*)L.u, L.parents, L.children)
   MAPGB_GEO_DISPATCH(kc, CALL_RES);
 #undef CALL_RES
 }
