@@ -200,34 +200,49 @@ __device__ __forceinline__ void load_global(const T* b, size_t S, int c, T* w) {
   for (int v = 0; v < NV; ++v) w[v] = b[(size_t)v * S + c];
 }
 
-// alpha_g: max over leaf interior cells and directions of |v_d| + c_f,d (Sec. 3.7).
+// alpha_g: max over leaf interior cells and directions of |v_d| + c_f,d (Sec. 3.7), one leaf
+// per CTA, two x-neighbours per thread (8-byte FP32 loads, two chains of roots).  The maxima
+// stay in T until one thread widens the leaf's for the atomic (a maximum is exact in any
+// precision, and widening is exact and monotone): FP64 on every warp, at 1/64 of the FP32
+// rate, had cost more than the cells of a 16^2 block.  32640 16^2 blocks: 228 us -> 63;
+// 256^3: 135 -> 106 (floor 89 and 44 us for one read of the state).
+template <int NDIM, int NB>
+__host__ __device__ constexpr int cfl_threads() {
+  constexpr int pairs = (NDIM == 3 ? NB * NB * NB : NB * NB) / 2;
+  return pairs < 128 ? pairs : 128;
+}
+
 template <typename T, int NDIM, int NB>
-__global__ void __launch_bounds__(256) cfl_kernel(const T* __restrict__ u, const int* __restrict__ blocks, int n,
-                                                  const BlockGeo* __restrict__ geo, ProbDyn* dyn, T gamma, T gm1,
-                                                  double kappa0) {
+__global__ void __launch_bounds__(cfl_threads<NDIM, NB>()) cfl_kernel(const T* __restrict__ u,
+                                                                      const int* __restrict__ blocks, int n,
+                                                                      const BlockGeo* __restrict__ geo, ProbDyn* dyn,
+                                                                      T gamma, T gm1, T kappa0) {
   using G = Geo<NDIM, NB>;
-  constexpr int NP = G::NP, S = G::S;
+  using V = Pack<T, 2>;
+  constexpr int NP = G::NP, S = G::S, NT = cfl_threads<NDIM, NB>();
   constexpr int NI = NDIM == 3 ? NB * NB * NB : NB * NB;
-  __shared__ double red[32], redk[32];
+  __shared__ T red[32], redk[32];
   Phys<T> P;
   P.gamma = gamma;
   P.gm1 = gm1;
   P.ch = T(0);
   P.tau = T(0);
+  const bool cond = kappa0 > T(0);
   chain_begin();
-  for (int bi = blockIdx.x; bi < n; bi += gridDim.x) {
-    const int blk = blocks[bi];
-    const T* ub = u + (size_t)blk * NV * S;
-    // maxima in T within each warp (a maximum is exact in any precision, and widening to
-    // FP64 is exact and monotone), then FP64 across warps
-    const bool cond = kappa0 > 0.0;
-    const T kap0 = (T)kappa0;
-    T am = T(0), km = T(0);
-    for (int c = threadIdx.x; c < NI; c += blockDim.x) {
-      const int i = c % NB, j = (c / NB) % NB, k = NDIM == 3 ? c / (NB * NB) : 0;
-      const int cc = ((NDIM == 3 ? k + NG : 0) * NP + j + NG) * NP + i + NG;
+  const int blk = blocks[blockIdx.x];
+  const T* ub = u + (size_t)blk * NV * S;
+  T am = T(0), km = T(0);
+  for (int c = 2 * threadIdx.x; c < NI; c += 2 * NT) {
+    const int i = c % NB, j = (c / NB) % NB, k = NDIM == 3 ? c / (NB * NB) : 0;
+    const T* cell = ub + ((NDIM == 3 ? k + NG : 0) * NP + j + NG) * NP + i + NG;
+    V q[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) q[v] = *reinterpret_cast<const V*>(cell + (size_t)v * S);
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
       T w[NV];
-      load_global<T>(ub, S, cc, w);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) w[v] = q[v].v[x];
       const T p = pressure<T>(w, P);
       T a = alpha_p<T, 0>(w, p, P);
       a = nan_max<T>(a, alpha_p<T, 1>(w, p, P));
@@ -236,29 +251,28 @@ __global__ void __launch_bounds__(256) cfl_kernel(const T* __restrict__ u, const
       if (cond) {
         // kappa T / p read as kappa / rho, kappa = kappa0 T^(5/2), T = max(p, 0) / rho
         const T tt = (p < T(0) ? T(0) : p) / w[RHO];
-        const T kr = kap0 * (tt * tt * sqrt(tt)) / w[RHO];
+        const T kr = kappa0 * (tt * tt * sqrt(tt)) / w[RHO];
         km = nan_max<T>(km, kr);
       }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      am = nan_max<T>(am, __shfl_xor_sync(0xffffffffu, am, o));
-      km = nan_max<T>(km, __shfl_xor_sync(0xffffffffu, km, o));
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    am = nan_max<T>(am, __shfl_xor_sync(0xffffffffu, am, o));
+    if (cond) km = nan_max<T>(km, __shfl_xor_sync(0xffffffffu, km, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[threadIdx.x >> 5] = am;
+    redk[threadIdx.x >> 5] = km;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < NT / 32; ++q) {
+      am = nan_max<T>(am, red[q]);
+      km = nan_max<T>(km, redk[q]);
     }
-    if ((threadIdx.x & 31) == 0) {
-      red[threadIdx.x >> 5] = (double)am;
-      redk[threadIdx.x >> 5] = (double)km;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double a = 0.0, kk = 0.0;
-      for (int q = 0; q < (int)(blockDim.x + 31) / 32; ++q) {
-        a = nan_max<double>(a, red[q]);
-        kk = nan_max<double>(kk, redk[q]);
-      }
-      atomicMax(&dyn[geo[blk].problem].alpha_bits, (unsigned long long)__double_as_longlong(a));
-      if (kappa0 > 0.0) atomicMax(&dyn[geo[blk].problem].kmax_bits, (unsigned long long)__double_as_longlong(kk));
-    }
-    __syncthreads();
+    ProbDyn* d = dyn + geo[blk].problem;
+    atomicMax(&d->alpha_bits, (unsigned long long)__double_as_longlong((double)am));
+    if (cond) atomicMax(&d->kmax_bits, (unsigned long long)__double_as_longlong((double)km));
   }
 }
 
