@@ -206,20 +206,29 @@ __device__ __forceinline__ void load_global(const T* b, size_t S, int c, T* w) {
 // precision, and widening is exact and monotone): FP64 on every warp, at 1/64 of the FP32
 // rate, had cost more than the cells of a 16^2 block.  32640 16^2 blocks: 228 us -> 63;
 // 256^3: 135 -> 106 (floor 89 and 44 us for one read of the state).
+//
+// A leaf goes to as many CTAs as give each thread four pairs (four for a 16^3 leaf): few
+// leaves then still reach every SM.  64 16^3 FP64 leaves, one CTA each: 200 us -> 103.
 template <int NDIM, int NB>
 __host__ __device__ constexpr int cfl_threads() {
   constexpr int pairs = (NDIM == 3 ? NB * NB * NB : NB * NB) / 2;
   return pairs < 128 ? pairs : 128;
 }
 
+template <int NDIM, int NB>
+__host__ __device__ constexpr int cfl_parts() {
+  constexpr int rounds = (NDIM == 3 ? NB * NB * NB : NB * NB) / 2 / cfl_threads<NDIM, NB>();
+  return rounds > 4 ? rounds / 4 : 1;
+}
+
 template <typename T, int NDIM, int NB>
 __global__ void __launch_bounds__(cfl_threads<NDIM, NB>()) cfl_kernel(const T* __restrict__ u,
-                                                                      const int* __restrict__ blocks, int n,
+                                                                      const int* __restrict__ blocks,
                                                                       const BlockGeo* __restrict__ geo, ProbDyn* dyn,
                                                                       T gamma, T gm1, T kappa0) {
   using G = Geo<NDIM, NB>;
   using V = Pack<T, 2>;
-  constexpr int NP = G::NP, S = G::S, NT = cfl_threads<NDIM, NB>();
+  constexpr int NP = G::NP, S = G::S, NT = cfl_threads<NDIM, NB>(), PARTS = cfl_parts<NDIM, NB>();
   constexpr int NI = NDIM == 3 ? NB * NB * NB : NB * NB;
   __shared__ T red[32], redk[32];
   Phys<T> P;
@@ -229,10 +238,10 @@ __global__ void __launch_bounds__(cfl_threads<NDIM, NB>()) cfl_kernel(const T* _
   P.tau = T(0);
   const bool cond = kappa0 > T(0);
   chain_begin();
-  const int blk = blocks[blockIdx.x];
+  const int blk = blocks[blockIdx.x / PARTS], part = blockIdx.x % PARTS;
   const T* ub = u + (size_t)blk * NV * S;
   T am = T(0), km = T(0);
-  for (int c = 2 * threadIdx.x; c < NI; c += 2 * NT) {
+  for (int c = part * (NI / PARTS) + 2 * threadIdx.x; c < (part + 1) * (NI / PARTS); c += 2 * NT) {
     const int i = c % NB, j = (c / NB) % NB, k = NDIM == 3 ? c / (NB * NB) : 0;
     const T* cell = ub + ((NDIM == 3 ? k + NG : 0) * NP + j + NG) * NP + i + NG;
     V q[NV];

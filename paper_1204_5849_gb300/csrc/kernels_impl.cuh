@@ -139,8 +139,8 @@ cudaError_t launch_cfl_T(const KernelConfig& kc, const CflLaunch& L, cudaStream_
   if (L.nblocks <= 0) return cudaSuccess;
   if (cnt) ++*cnt;
 #define CALL_CFL(ND, NBV)                                                                     \
-  return launch_chained(cfl_kernel<T, ND, NBV>, L.nblocks, cfl_threads<ND, NBV>(), 0, s, (const T*)L.u, L.blocks, \
-                        L.nblocks, L.geo, L.dyn, (T)L.gamma, (T)(L.gamma - 1.0), (T)L.kappa0)
+  return launch_chained(cfl_kernel<T, ND, NBV>, L.nblocks * cfl_parts<ND, NBV>(), cfl_threads<ND, NBV>(), 0, s, \
+                        (const T*)L.u, L.blocks, L.geo, L.dyn, (T)L.gamma, (T)(L.gamma - 1.0), (T)L.kappa0)
   MAPGB_GEO_DISPATCH(kc, CALL_CFL);
 #undef CALL_CFL
 }
