@@ -575,72 +575,57 @@ __global__ void __launch_bounds__(256) regrid_kernel(RegridLaunch L) {
 // step kernel is replaced by the mean of the fine fluxes covering the cell:
 //   u_c += lam (F_fine - F_coarse) on a low face, u_c -= lam (F_fine - F_coarse) on a high one
 // (lam = dt / dx_d of the coarse leaf; psi's correction carries the damping factor the step
-// already applied).  Faces go in the order (d, low then high) with a barrier between them, so a
-// cell on two such faces is corrected in a fixed order.  Then every corrected cell is checked
-// and stored again into the ghost regions of the same-level leaves that copy it, and, in the
-// fused form, added to alpha_g and the FP64 sums (the step kernel left these cells out).
+// already applied).  A thread takes a corrected cell: it applies the faces the cell lies on in
+// the order (d, low then high), checks the cell, stores it again into the ghost regions of the
+// same-level leaves that copy it and, in the fused form, adds it to alpha_g and the FP64 sums
+// (the step kernel left these cells out).
+//
+// The kernel is bound by latency -- a few hundred cells per leaf, each a chain of register
+// loads -- and by FP64, at 1/64 of the FP32 rate: so no face waits for another, dt/dx is one
+// division on one warp, and the sums of a warp are reduced by halving the number of variables
+// with the number of lanes that hold them (16 additions instead of 45).  Faces one after the
+// other with a barrier each, and every sum through all lanes: 27 -> 15 us per launch on the
+// rotor's quadtree (16^2), 57 -> 26 on a 9472-leaf octree (8^3).
+template <int NDIM, int NB>
+__host__ __device__ constexpr int reflux_threads() {
+  return NDIM == 2 ? 64 : (NB == 8 ? 192 : 256);
+}
+
 template <typename T, int NDIM, int NB>
-__global__ void __launch_bounds__(256) reflux_kernel(RefluxLaunch L) {
+__global__ void __launch_bounds__(reflux_threads<NDIM, NB>()) reflux_kernel(RefluxLaunch L) {
   using G = Geo<NDIM, NB>;
-  constexpr int NP = G::NP, S = G::S;
+  constexpr int NP = G::NP, S = G::S, NT = reflux_threads<NDIM, NB>(), NW = NT / 32;
   constexpr int NF = NDIM == 3 ? NB * NB : NB;          // face cells per face
   constexpr int H = NB / 2;
   constexpr size_t NB2 = (size_t)NB * NB;
   constexpr size_t PER = (size_t)2 * NDIM * NV * NB2;   // one register slot
-  __shared__ double red[NV + 1][32];
+  __shared__ double red[NV + 1][NW];
+  __shared__ T lam_s[3];
+  __shared__ RefluxTask tk;
   chain_begin();
-  const RefluxTask& tk = L.tasks[blockIdx.x];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  {
+    constexpr int words = sizeof(RefluxTask) / sizeof(int);
+    static_assert(sizeof(RefluxTask) % sizeof(int) == 0 && words <= 32, "one word per lane");
+    if (tid < words) reinterpret_cast<int*>(&tk)[tid] = reinterpret_cast<const int*>(L.tasks + blockIdx.x)[tid];
+  }
+  __syncthreads();
   const int q = tk.coarse;
-  const BlockGeo gg = L.geo[q];
-  const ProbDyn dy = L.dyn[gg.problem];
+  const int prob = L.geo[q].problem;
+  if (L.nsub && L.it >= L.nsub[prob]) return;              // no substep for this problem
+  if (wid == 0) {
+    const double dtp = L.hsub ? L.hsub[prob] : L.dyn[prob].dt;
+    const double l = dtp / L.geo[q].dx[lane < NDIM ? lane : 0];
+    if (lane < NDIM) lam_s[lane] = (T)l;
+  }
+  __syncthreads();
   T* ub = (T*)L.u + (size_t)q * NV * S;
   const T* freg = (const T*)L.freg;
-  const T damp = (T)dy.damp;
+  const T damp = (T)L.dyn[prob].damp;
   int mask = 0;
+#pragma unroll
   for (int f = 0; f < 2 * NDIM; ++f)
     if (tk.fslot[f][0] >= 0) mask |= 1 << f;
-  // padded offset of the coarse cell on face (d, side) at face cell (t0, t1)
-  auto cell_of = [&](int d, int side, int t0, int t1, int* ci) {
-    const int da = d == 0 ? 1 : 0, db = d == 2 ? 1 : 2;
-    ci[0] = ci[1] = ci[2] = 0;
-    ci[d] = side ? NB - 1 : 0;
-    ci[da] = t0;
-    if (NDIM == 3) ci[db] = t1;
-    return ((NDIM == 3 ? ci[2] + NG : 0) * NP + ci[1] + NG) * NP + ci[0] + NG;
-  };
-  if (L.nsub && L.it >= L.nsub[gg.problem]) return;        // no substep for this problem
-  const double dtp = L.hsub ? L.hsub[gg.problem] : dy.dt;
-  for (int d = 0; d < NDIM; ++d)
-    for (int side = 0; side < 2; ++side) {
-      const int f = 2 * d + side;
-      if (!((mask >> f) & 1)) continue;
-      const T lam = (T)(dtp / gg.dx[d]);
-      const T* rc = freg + (size_t)tk.cslot * PER + (size_t)f * NV * NB2;
-      for (int idx = threadIdx.x; idx < NF; idx += blockDim.x) {
-        const int t0 = idx % NB, t1 = NDIM == 3 ? idx / NB : 0;
-        const int k = t0 / H + (NDIM == 3 ? 2 * (t1 / H) : 0);
-        const T* rf = freg + (size_t)tk.fslot[f][k] * PER + (size_t)(2 * d + 1 - side) * NV * NB2;
-        const int f0 = 2 * (t0 - (t0 / H) * H), f1 = NDIM == 3 ? 2 * (t1 - (t1 / H) * H) : 0;
-        int ci[3];
-        const int c = cell_of(d, side, t0, t1, ci);
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          if (v < L.v0 || v >= L.v1) continue;
-          const T* fv = rf + (size_t)v * NB2;
-          T ff;
-          if (NDIM == 2) ff = T(0.5) * (fv[f0] + fv[f0 + 1]);
-          else ff = T(0.25) * ((fv[f1 * NB + f0] + fv[f1 * NB + f0 + 1]) +
-                               (fv[(f1 + 1) * NB + f0] + fv[(f1 + 1) * NB + f0 + 1]));
-          T corr = lam * (ff - rc[(size_t)v * NB2 + t1 * NB + t0]);
-          if (v == PSI) corr = corr * damp;
-          T* cell = ub + (size_t)v * S + c;
-          *cell = side ? *cell - corr : *cell + corr;
-        }
-      }
-      __syncthreads();
-    }
-  // checks, pushes and fused diagnostics, once per corrected cell (a cell on several such
-  // faces is taken with the first of them)
   Phys<T> P;
   P.gamma = (T)L.gamma;
   P.gm1 = (T)(L.gamma - 1.0);
@@ -651,91 +636,133 @@ __global__ void __launch_bounds__(256) reflux_kernel(RefluxLaunch L) {
   double sum[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) sum[v] = 0.0;
-  for (int d = 0; d < NDIM; ++d)
-    for (int side = 0; side < 2; ++side) {
-      const int f = 2 * d + side;
-      if (!((mask >> f) & 1)) continue;
-      for (int idx = threadIdx.x; idx < NF; idx += blockDim.x) {
-        const int t0 = idx % NB, t1 = NDIM == 3 ? idx / NB : 0;
-        int ci[3];
-        const int c = cell_of(d, side, t0, t1, ci);
-        bool first = true;
-        for (int f2 = 0; f2 < f; ++f2)
-          if (((mask >> f2) & 1) && ci[f2 >> 1] == ((f2 & 1) ? NB - 1 : 0)) first = false;
-        if (!first) continue;
-        T w[NV];
+  for (int item = tid; item < __popc(mask) * NF; item += NT) {
+    int f = 0, rank = item / NF;                           // the face of this item: the rank-th in the mask
 #pragma unroll
-        for (int v = 0; v < NV; ++v) w[v] = ub[(size_t)v * S + c];
-        bool fin = true;
+    for (int f2 = 0; f2 < 2 * NDIM; ++f2)
+      if ((mask >> f2) & 1) {
+        if (rank == 0) f = f2;
+        --rank;
+      }
+    const int d0 = f >> 1, s0 = f & 1, idx = item % NF;
+    int ci[3] = {0, 0, 0};
+    {
+      const int t0 = idx % NB, t1 = NDIM == 3 ? idx / NB : 0;
+      ci[0] = d0 == 0 ? (s0 ? NB - 1 : 0) : t0;
+      ci[1] = d0 == 1 ? (s0 ? NB - 1 : 0) : (d0 == 0 ? t0 : t1);
+      ci[2] = NDIM == 3 ? (d0 == 2 ? (s0 ? NB - 1 : 0) : t1) : 0;
+    }
+    // a cell on several such faces is taken with the first of them
+    bool first = true;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) fin = fin && isfinite(w[v]);
-        if (!fin) {
-          errbits |= 1u;
-          am = (T)NAN;
-        } else {
-          const T pr = pressure<T>(w, P);
-          if (!(w[RHO] > T(0)) || pr < T(0)) errbits |= 2u;
-          T a = alpha_p<T, 0>(w, pr, P);
-          a = dmax<T>(a, alpha_p<T, 1>(w, pr, P));
-          if (NDIM == 3) a = dmax<T>(a, alpha_p<T, 2>(w, pr, P));
-          if (!(am != am)) am = dmax<T>(am, a);
+    for (int f2 = 0; f2 < 2 * NDIM; ++f2)
+      if (f2 < f && ((mask >> f2) & 1) && ci[f2 >> 1] == ((f2 & 1) ? NB - 1 : 0)) first = false;
+    if (!first) continue;
+    const int c = ((NDIM == 3 ? ci[2] + NG : 0) * NP + ci[1] + NG) * NP + ci[0] + NG;
+    T w[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) w[v] = ub[(size_t)v * S + c];
+#pragma unroll
+    for (int d = 0; d < NDIM; ++d) {
+      const int t0 = d == 0 ? ci[1] : ci[0], t1 = NDIM == 3 ? (d == 2 ? ci[1] : ci[2]) : 0;
+      const int k = t0 / H + (NDIM == 3 ? 2 * (t1 / H) : 0);
+      const int f0 = 2 * (t0 % H), f1 = NDIM == 3 ? 2 * (t1 % H) : 0;
+#pragma unroll
+      for (int side = 0; side < 2; ++side) {
+        const int fs = 2 * d + side;
+        if (!((mask >> fs) & 1) || ci[d] != (side ? NB - 1 : 0)) continue;
+        const T* rc = freg + (size_t)tk.cslot * PER + (size_t)fs * NV * NB2 + t1 * NB + t0;
+        const T* rf = freg + (size_t)tk.fslot[fs][k] * PER + (size_t)(2 * d + 1 - side) * NV * NB2 + f1 * NB + f0;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          if (v < L.v0 || v >= L.v1) continue;
+          const T* fv = rf + (size_t)v * NB2;
+          T ff;
+          if (NDIM == 2) ff = T(0.5) * (fv[0] + fv[1]);
+          else ff = T(0.25) * ((fv[0] + fv[1]) + (fv[NB] + fv[NB + 1]));
+          T corr = lam_s[d] * (ff - rc[(size_t)v * NB2]);
+          if (v == PSI) corr = corr * damp;
+          w[v] = side ? w[v] - corr : w[v] + corr;
         }
-#pragma unroll
-        for (int v = 0; v < NV; ++v) sum[v] += (double)w[v];
-        // the same-level leaves that copy this cell into their ghosts
-        const int x = ci[0] + NG, y = ci[1] + NG, z = NDIM == 3 ? ci[2] + NG : 0;
-        const int fx = x < 2 * NG ? -1 : (x >= NB ? 1 : 0);
-        const int fy = y < 2 * NG ? -1 : (y >= NB ? 1 : 0);
-        const int fz = NDIM == 3 ? (z < 2 * NG ? -1 : (z >= NB ? 1 : 0)) : 0;
-        for (int kz = 0; kz < (fz ? 2 : 1); ++kz)
-          for (int ky = 0; ky < (fy ? 2 : 1); ++ky)
-            for (int kx = 0; kx < (fx ? 2 : 1); ++kx) {
-              const int ex = kx ? fx : 0, ey = ky ? fy : 0, ez = kz ? fz : 0;
-              if (!(ex | ey | ez)) continue;
-              const PushEntry pe = L.pushes[(size_t)q * 27 + (ex + 1) + 3 * (ey + 1) + 9 * (ez + 1)];
-              if (pe.dst < 0) continue;
-              T* db = (T*)L.u + (size_t)pe.dst * NV * S;
-              const size_t dc = ((size_t)(z + pe.off[2]) * NP + (y + pe.off[1])) * NP + (x + pe.off[0]);
-#pragma unroll
-              for (int v = 0; v < NV; ++v) db[(size_t)v * S + dc] = w[v];
-            }
       }
     }
+    bool fin = true;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      if (v >= L.v0 && v < L.v1) ub[(size_t)v * S + c] = w[v];
+      fin = fin && isfinite(w[v]);
+    }
+    if (!fin) {
+      errbits |= 1u;
+      am = (T)NAN;
+    } else {
+      const T pr = pressure<T>(w, P);
+      if (!(w[RHO] > T(0)) || pr < T(0)) errbits |= 2u;
+      if (L.dyn_next) {
+        T a = alpha_p<T, 0>(w, pr, P);
+        a = dmax<T>(a, alpha_p<T, 1>(w, pr, P));
+        if (NDIM == 3) a = dmax<T>(a, alpha_p<T, 2>(w, pr, P));
+        if (!(am != am)) am = dmax<T>(am, a);
+      }
+    }
+    if (L.sums) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) sum[v] += (double)w[v];
+    }
+    // the same-level leaves that copy this cell into their ghosts
+    const int x = ci[0] + NG, y = ci[1] + NG, z = NDIM == 3 ? ci[2] + NG : 0;
+    const int fx = x < 2 * NG ? -1 : (x >= NB ? 1 : 0);
+    const int fy = y < 2 * NG ? -1 : (y >= NB ? 1 : 0);
+    const int fz = NDIM == 3 ? (z < 2 * NG ? -1 : (z >= NB ? 1 : 0)) : 0;
+    for (int kz = 0; kz < (fz ? 2 : 1); ++kz)
+      for (int ky = 0; ky < (fy ? 2 : 1); ++ky)
+        for (int kx = 0; kx < (fx ? 2 : 1); ++kx) {
+          const int ex = kx ? fx : 0, ey = ky ? fy : 0, ez = kz ? fz : 0;
+          if (!(ex | ey | ez)) continue;
+          const PushEntry pe = L.pushes[(size_t)q * 27 + (ex + 1) + 3 * (ey + 1) + 9 * (ez + 1)];
+          if (pe.dst < 0) continue;
+          T* db = (T*)L.u + (size_t)pe.dst * NV * S;
+          const size_t dc = ((size_t)(z + pe.off[2]) * NP + (y + pe.off[1])) * NP + (x + pe.off[0]);
+#pragma unroll
+          for (int v = 0; v < NV; ++v) db[(size_t)v * S + dc] = w[v];
+        }
+  }
   unsigned e = errbits;
   for (int o = 16; o > 0; o >>= 1) e |= __shfl_xor_sync(0xffffffffu, e, o);
-  if ((threadIdx.x & 31) == 0 && e) atomicOr(L.err_word, e);
+  if (lane == 0 && e) atomicOr(L.err_word, e);
   if (!L.dyn_next && !L.sums) return;
-  double a2 = (double)am;
-  for (int o = 16; o > 0; o >>= 1) {
-    const double t = __shfl_xor_sync(0xffffffffu, a2, o);
-    a2 = (t != t || a2 != a2) ? __longlong_as_double(0x7ff8000000000000ll) : fmax(a2, t);
-  }
+  for (int o = 16; o > 0; o >>= 1) am = nan_max<T>(am, __shfl_xor_sync(0xffffffffu, am, o));
+  // the warp's sums of sixteen values (nine in use): after the exchange over lane bit b a lane
+  // keeps the half of its values whose index agrees with that bit, so lanes v and v + 16 end
+  // with the halves of value v
+  double s[16];
 #pragma unroll
-  for (int v = 0; v < NV; ++v)
-    for (int o = 16; o > 0; o >>= 1) sum[v] += __shfl_xor_sync(0xffffffffu, sum[v], o);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) {
-    red[NV][wid] = a2;
+  for (int v = 0; v < 16; ++v) s[v] = v < NV ? sum[v < NV ? v : 0] : 0.0;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) red[v][wid] = sum[v];
+  for (int b = 3; b >= 0; --b) {
+    const int half = 1 << b;
+    const bool up = (lane >> b) & 1;
+#pragma unroll
+    for (int v = 0; v < half; ++v) {
+      const double give = up ? s[v] : s[v + half], keep = up ? s[v + half] : s[v];
+      s[v] = keep + __shfl_xor_sync(0xffffffffu, give, half);
+    }
   }
+  s[0] += __shfl_xor_sync(0xffffffffu, s[0], 16);
+  if (lane < NV) red[lane][wid] = s[0];
+  if (lane == NV) red[NV][wid] = (double)am;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const int nw = (blockDim.x + 31) / 32;
+  if (tid == NV && L.dyn_next) {
     double a = 0.0;
-    for (int w2 = 0; w2 < nw; ++w2) {
-      const double t = red[NV][w2];
-      a = (t != t || a != a) ? __longlong_as_double(0x7ff8000000000000ll) : fmax(a, t);
-    }
-    if (L.dyn_next) atomicMax(&L.dyn_next[gg.problem].alpha_bits, (unsigned long long)__double_as_longlong(a));
-    if (L.sums) {
-      const double vol = gg.dx[0] * gg.dx[1] * (NDIM == 3 ? gg.dx[2] : 1.0);
-      for (int v = 0; v < NV; ++v) {
-        double t = 0.0;
-        for (int w2 = 0; w2 < nw; ++w2) t += red[v][w2];
-        atomicAdd(&L.sums[gg.problem * NV + v], t * vol);
-      }
-    }
+    for (int k = 0; k < NW; ++k) a = nan_max<double>(a, red[NV][k]);
+    atomicMax(&L.dyn_next[prob].alpha_bits, (unsigned long long)__double_as_longlong(a));
+  }
+  if (tid < NV && L.sums) {
+    const BlockGeo gg = L.geo[q];
+    const double vol = gg.dx[0] * gg.dx[1] * (NDIM == 3 ? gg.dx[2] : 1.0);
+    double t = 0.0;
+    for (int k = 0; k < NW; ++k) t += red[tid][k];
+    atomicAdd(&L.sums[prob * NV + tid], t * vol);
   }
 }
 

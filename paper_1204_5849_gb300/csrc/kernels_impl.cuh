@@ -213,7 +213,7 @@ cudaError_t launch_reflux_T(const KernelConfig& kc, const RefluxLaunch& L, cudaS
   if (L.ntasks <= 0) return cudaSuccess;
   if (cnt) ++*cnt;
 #define CALL_REFLUX(ND, NBV)                                              \
-  return launch_chained(reflux_kernel<T, ND, NBV>, L.ntasks, 256, 0, s, L)
+  return launch_chained(reflux_kernel<T, ND, NBV>, L.ntasks, reflux_threads<ND, NBV>(), 0, s, L)
   MAPGB_GEO_DISPATCH(kc, CALL_REFLUX);
 #undef CALL_REFLUX
 }
