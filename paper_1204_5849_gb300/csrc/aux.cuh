@@ -325,27 +325,31 @@ __global__ void __launch_bounds__(256) cfl_partial_kernel(const T* __restrict__ 
   }
 }
 
-// Refinement estimator (Sec. 4.5), computed in FP64 from the pool values, over the
-// interior and the first ghost ring; block maximum -> flag.
+// Refinement estimator (Sec. 4.5) in the pool's precision, over the interior and the first
+// ghost ring; block maximum -> flag.  The parameters come rounded to that precision (FlagArgs)
+// and one thread rounds the leaf's spacings: FP64 operations and conversions on every thread,
+// at 1/64 of the FP32 rate, had kept an FP32 pool's kernel on the FP64 pipe (84 % busy).
+// 9472 8^3 leaves, |J| criterion: 176 -> 66 us.
 template <typename T, int NDIM, int NB>
-__global__ void __launch_bounds__(256) flags_kernel(FlagLaunch L) {
+__global__ void __launch_bounds__(256) flags_kernel(FlagArgs<T> L) {
   // the estimator runs in the pool's precision: FP64 pools bitwise as the FP64 formula, FP32
   // pools in FP32 (decisions then differ from FP64 only within float rounding of a threshold)
   using R = T;
   using G = Geo<NDIM, NB>;
   constexpr int NP = G::NP, P2 = G::P2, S = G::S;
   constexpr int NR = NDIM == 3 ? (NB + 2) * (NB + 2) * (NB + 2) : (NB + 2) * (NB + 2);
-  __shared__ double red[32];
-  const T* u = (const T*)L.u;
-  const R gm1 = (R)(L.gamma - 1.0);
-  const R bias = (R)L.r.bias, filt = (R)L.r.filter;
+  __shared__ R red[32];
+  __shared__ R two_dx[3];
+  __shared__ R mindx_s;
+  const T* u = L.u;
+  const R bias = L.bias, filt = L.filter;
   const R half_sqrt3 = (R)(1.7320508075688772 / 2.0);
   // the pool's pressure recovery (FP32 pools: with its FP64 fallback at low e_int / e)
   Phys<T> PP;
-  PP.gamma = (T)L.gamma;
-  PP.gm1 = (T)gm1;
+  PP.gamma = L.gamma;
+  PP.gm1 = L.gm1;
   PP.ch = T(0);
-  PP.tau = (T)L.tau;
+  PP.tau = L.tau;
   auto pres = [&](const T* ub, int c) -> R {
     R w[NV];
 #pragma unroll
@@ -355,12 +359,21 @@ __global__ void __launch_bounds__(256) flags_kernel(FlagLaunch L) {
   const int offs[3] = {1, NP, P2};
   for (int bi = blockIdx.x; bi < L.nblocks; bi += gridDim.x) {
     const int blk = L.blocks[bi];
-    const BlockGeo gg = L.geo[blk];
+    const int level = L.geo[blk].level;
     const T* ub = u + (size_t)blk * NV * S;
-    double mindx = gg.dx[0];
-    for (int d = 1; d < NDIM; ++d) mindx = fmin(mindx, gg.dx[d]);
-    const R lvf = (R)L.level_factor[gg.level < 16 ? gg.level : 15];
-    const R two_dx[3] = {(R)(2.0 * gg.dx[0]), (R)(2.0 * gg.dx[1]), (R)(NDIM == 3 ? 2.0 * gg.dx[2] : 1.0)};
+    if (threadIdx.x == 0) {
+      const BlockGeo gg = L.geo[blk];
+      R least = (R)gg.dx[0];                       // rounding keeps the order
+      for (int d = 0; d < 3; ++d) {
+        const R dx = (R)gg.dx[d];
+        two_dx[d] = d < NDIM ? R(2) * dx : R(1);   // doubling is exact
+        if (d < NDIM) least = fmin(least, dx);
+      }
+      mindx_s = least;
+    }
+    __syncthreads();
+    const R mindx = mindx_s;
+    const R lvf = L.level_factor[level < 16 ? level : 15];
     R emax = R(0);
     for (int q = threadIdx.x; q < NR; q += blockDim.x) {
       const int i = 1 + q % (NB + 2), j = 1 + (q / (NB + 2)) % (NB + 2);
@@ -382,9 +395,9 @@ __global__ void __launch_bounds__(256) flags_kernel(FlagLaunch L) {
         const R e = bias * du / au + (R(1) - bias) * d2u / (du + filt * au);
         return e * lvf;
       };
-      if (L.r.var_mask & 1) emax = fmax(emax, est([&](int cc) { return (R)ub[RHO * (size_t)S + cc]; }, (R)L.r.eps_rho));
-      if (L.r.var_mask & 2) emax = fmax(emax, est([&](int cc) { return pres(ub, cc); }, (R)L.r.eps_p));
-      if (L.r.var_mask & 4) {
+      if (L.var_mask & 1) emax = fmax(emax, est([&](int cc) { return (R)ub[RHO * (size_t)S + cc]; }, L.eps_rho));
+      if (L.var_mask & 2) emax = fmax(emax, est([&](int cc) { return pres(ub, cc); }, L.eps_p));
+      if (L.var_mask & 4) {
         auto cd = [&](int comp, int d) -> R {
           if (d >= NDIM) return R(0);
           return ((R)ub[(size_t)comp * S + c + offs[d]] - (R)ub[(size_t)comp * S + c - offs[d]]) / two_dx[d];
@@ -393,20 +406,20 @@ __global__ void __launch_bounds__(256) flags_kernel(FlagLaunch L) {
         const R jy = cd(BX, 2) - cd(BZ, 0);
         const R jz = cd(BY, 0) - cd(BX, 1);
         const R bx = ub[(size_t)BX * S + c], by = ub[(size_t)BY * S + c], bz = ub[(size_t)BZ * S + c];
-        const R e = sqrt(jx * jx + jy * jy + jz * jz) * (R)mindx / (sqrt(bx * bx + by * by + bz * bz) + (R)L.r.eps_b);
+        const R e = sqrt(jx * jx + jy * jy + jz * jz) * mindx / (sqrt(bx * bx + by * by + bz * bz) + L.eps_b);
         emax = fmax(emax, e);
       }
     }
-    double em = (double)emax;
-    for (int o = 16; o > 0; o >>= 1) em = fmax(em, __shfl_xor_sync(0xffffffffu, em, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = em;
+    for (int o = 16; o > 0; o >>= 1) emax = fmax(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = emax;
     __syncthreads();
     if (threadIdx.x == 0) {
-      double e = 0.0;
-      for (int q = 0; q < (int)(blockDim.x + 31) / 32; ++q) e = fmax(e, red[q]);
+      R er = R(0);
+      for (int q = 0; q < (int)(blockDim.x + 31) / 32; ++q) er = fmax(er, red[q]);
+      const double e = (double)er;
       int8_t f = 0;
-      if (e > L.r.thr && gg.level < L.r.max_level) f = 1;
-      else if (e < L.r.coarsen_thr && gg.level > 0) f = -1;
+      if (e > L.thr && level < L.max_level) f = 1;
+      else if (e < L.coarsen_thr && level > 0) f = -1;
       L.flags[bi] = f;
       if (L.est) L.est[bi] = e;
     }

@@ -150,7 +150,7 @@ cudaError_t launch_flags_T(const KernelConfig& kc, const FlagLaunch& L, cudaStre
   if (L.nblocks <= 0) return cudaSuccess;
   if (cnt) ++*cnt;
 #define CALL_FLAGS(ND, NBV)                                              \
-  flags_kernel<T, ND, NBV><<<grid_for(L.nblocks), 256, 0, s>>>(L);       \
+  flags_kernel<T, ND, NBV><<<grid_for(L.nblocks), 256, 0, s>>>(FlagArgs<T>(L)); \
   return cudaGetLastError()
   MAPGB_GEO_DISPATCH(kc, CALL_FLAGS);
 #undef CALL_FLAGS

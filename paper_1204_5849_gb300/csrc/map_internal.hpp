@@ -290,6 +290,28 @@ struct FlagLaunch {
   double level_factor[16];   // R^(xi (L+1-1)) for levels L = 0..15, computed on the host
 };
 
+// FlagLaunch with the estimator's parameters rounded to the pool's precision
+template <typename T>
+struct FlagArgs {
+  explicit FlagArgs(const FlagLaunch& l)
+      : u((const T*)l.u), blocks(l.blocks), nblocks(l.nblocks), geo(l.geo), gamma((T)l.gamma), gm1((T)(l.gamma - 1.0)),
+        tau((T)l.tau), bias((T)l.r.bias), filter((T)l.r.filter), eps_rho((T)l.r.eps_rho), eps_p((T)l.r.eps_p),
+        eps_b((T)l.r.eps_b), thr(l.r.thr), coarsen_thr(l.r.coarsen_thr), var_mask(l.r.var_mask),
+        max_level(l.r.max_level), flags(l.flags), est(l.est) {
+    for (int q = 0; q < 16; ++q) level_factor[q] = (T)l.level_factor[q];
+  }
+  const T* u;
+  const int* blocks;
+  int nblocks;
+  const BlockGeo* geo;
+  T gamma, gm1, tau, bias, filter, eps_rho, eps_p, eps_b;
+  double thr, coarsen_thr;
+  int var_mask, max_level;
+  int8_t* flags;
+  double* est;
+  T level_factor[16];
+};
+
 struct SumLaunch {
   const void* u;
   const int* blocks;
