@@ -791,60 +791,112 @@ __global__ void __launch_bounds__(reflux_threads<NDIM, NB>()) reflux_kernel(Refl
 // through their own ghost copies, so the in-place write is safe.  Boundary face fluxes go to
 // the face register's energy slot as fluxes of e along +d (-F) for reflux.
 
+// Products that are not contracted into a sum, so that both conduction kernels round alike
+// wherever the compiler would fuse one of them differently; quotients by a fixed b likewise: the
+// plain quotient in FP64, the product with the reciprocal rb = qdiv(1, b) in FP32.
+__device__ __forceinline__ float pmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double pmul(double a, double b) { return a * b; }
+__device__ __forceinline__ float pquo(float a, float, float rb) { return __fmul_rn(a, rb); }
+__device__ __forceinline__ double pquo(double a, double b, double) { return a / b; }
+
+// pressure<T> with every rounding spelled out, for the same reason (the loop keeps the parts
+// of it that conduction leaves alone, which no product may be fused across)
+__device__ __forceinline__ double cond_pressure(const double* w, const Phys<double>& P) { return pressure<double>(w, P); }
+__device__ __forceinline__ float cond_pressure(const float* w, const Phys<float>& P) {
+  const float m2 = __fmaf_rn(w[MZ], w[MZ], __fmaf_rn(w[MY], w[MY], __fmul_rn(w[MX], w[MX])));
+  const float b2 = __fmaf_rn(w[BZ], w[BZ], __fmaf_rn(w[BY], w[BY], __fmul_rn(w[BX], w[BX])));
+  const float kin = __fmul_rn(0.5f * m2, qdiv(1.0f, w[RHO]));
+  const float eint = __fadd_rn(__fadd_rn(w[EN], -kin), -0.5f * b2);
+  if (eint < P.tau * w[EN]) return pressure_fp64(w[RHO], w[MX], w[MY], w[MZ], w[BX], w[BY], w[BZ], w[EN], P.gm1);
+  return __fmul_rn(P.gm1, eint);
+}
+
 // T and kappa of one cell from its state
 template <typename T>
 __device__ __forceinline__ void cond_tk(const T* w, const Phys<T>& P, T k0, T& tt, T& kk) {
-  T p = pressure<T>(w, P);
+  T p = cond_pressure(w, P);
   if (p < T(0)) p = T(0);
-  tt = p / w[RHO];
-  kk = k0 * (tt * tt * sqrt(tt));
+  tt = pquo(p, w[RHO], sizeof(T) == 4 ? qdiv<T>(T(1), w[RHO]) : T(0));
+  kk = pmul(k0, pmul(pmul(tt, tt), sqrt(tt)));
 }
 
+// The two faces of a cell in direction d: their mean field and |B|^2 (unused for the isotropic
+// form), which conduction leaves as they are.
+template <typename T>
+struct CondFaces {
+  T b[2][3], b2[2];
+};
+
+// B: the three components, S apart; c: the cell's index; po: the stride of direction d
+template <typename T>
+__device__ __forceinline__ void cond_faces(const T* B, size_t S, int c, int po, CondFaces<T>& f) {
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    const int cl = side ? c : c - po, cr = cl + po;
+    f.b2[side] = T(0);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      f.b[side][j] = pmul(T(0.5), B[(size_t)j * S + cl] + B[(size_t)j * S + cr]);
+      f.b2[side] += pmul(f.b[side][j], f.b[side][j]);
+    }
+  }
+}
+
+// Spacings of a leaf in T, with their reciprocals and those of twice the spacing.
+template <typename T>
+struct CondDx {
+  T dx[3], rdx[3], rdx2[3];
+  __device__ __forceinline__ explicit CondDx(const BlockGeo& g) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      dx[d] = (T)g.dx[d];
+      rdx[d] = sizeof(T) == 4 ? qdiv<T>(T(1), dx[d]) : T(0);
+      rdx2[d] = T(0.5) * rdx[d];
+    }
+  }
+};
+
 // The energy rate of one interior cell: r its ring-region index (strides ro), sT / sK the
-// ring's T and kappa, bmean(j, d, side) the face mean of B_j on face side of direction d,
-// face(d, F) sees the two face fluxes of direction d (the reflux registers take them).  Both
-// conduction kernels call it, so their arithmetic is the same.
-template <typename T, int NDIM, typename BM, typename FF>
-__device__ __forceinline__ T cond_rate(const T* sT, const T* sK, int r, const int* ro, const BlockGeo& gg,
-                                       T gmax, int mode, BM bmean, FF face) {
+// ring's T and kappa, faces(d) the faces of direction d, face(d, F) sees their two fluxes (the
+// reflux registers take them).  Both conduction kernels call it, so their arithmetic is the
+// same.
+template <typename T, int NDIM, typename BF, typename FF>
+__device__ __forceinline__ T cond_rate(const T* sT, const T* sK, int r, const int* ro, const CondDx<T>& X,
+                                       T gmax, int mode, BF faces, FF face) {
   T acc = T(0);
 #pragma unroll
   for (int d = 0; d < NDIM; ++d) {
     T F[2];
+    const CondFaces<T> cf = faces(d);
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
       const int rl = side ? r : r - ro[d], rr = rl + ro[d];
-      T gn = (sT[rr] - sT[rl]) / (T)gg.dx[d];
+      T gn = pquo(sT[rr] - sT[rl], X.dx[d], X.rdx[d]);
       if (gmax > T(0)) gn = fmax(-gmax, fmin(gmax, gn));
-      const T kf = sqrt(sK[rl] * sK[rr]);
+      const T kf = sqrt(pmul(sK[rl], sK[rr]));
       if (mode == 1) {
-        F[side] = kf * gn;
+        F[side] = pmul(kf, gn);
       } else {
-        T bf[3], b2 = T(0);
-#pragma unroll
-        for (int j2 = 0; j2 < 3; ++j2) {
-          bf[j2] = bmean(j2, d, side);
-          b2 += bf[j2] * bf[j2];
-        }
+        const T* bf = cf.b[side];
+        const T b2 = cf.b2[side];
         if (!(b2 > T(0))) {
           F[side] = T(0);
         } else {
-          T bg = bf[d] * gn;
+          T bg = pmul(bf[d], gn);
 #pragma unroll
           for (int t = 0; t < NDIM; ++t) {
             if (t == d) continue;
-            const T dxt = (T)gg.dx[t];
-            T gt = T(0.5) * ((sT[rl + ro[t]] - sT[rl - ro[t]]) / (T(2) * dxt) +
-                             (sT[rr + ro[t]] - sT[rr - ro[t]]) / (T(2) * dxt));
+            T gt = pmul(T(0.5), pquo(sT[rl + ro[t]] - sT[rl - ro[t]], T(2) * X.dx[t], X.rdx2[t]) +
+                                    pquo(sT[rr + ro[t]] - sT[rr - ro[t]], T(2) * X.dx[t], X.rdx2[t]));
             if (gmax > T(0)) gt = fmax(-gmax, fmin(gmax, gt));
-            bg += bf[t] * gt;
+            bg += pmul(bf[t], gt);
           }
-          F[side] = kf * bf[d] * bg / b2;
+          F[side] = qdiv<T>(pmul(pmul(kf, bf[d]), bg), b2);
         }
       }
     }
     face(d, F);
-    acc += (F[1] - F[0]) / (T)gg.dx[d];
+    acc += pquo(F[1] - F[0], X.dx[d], X.rdx[d]);
   }
   return acc;
 }
@@ -885,14 +937,16 @@ __global__ void __launch_bounds__(256) conduction_kernel(CondLaunch L) {
   T* R0 = slot >= 0 ? (T*)L.freg + (size_t)slot * (2 * NDIM * NV * NB2) : nullptr;
   const int ro[3] = {1, R, R * R};
   const int po[3] = {1, NP, NP * NP};
+  const CondDx<T> X(gg);
   for (int q = threadIdx.x; q < NI; q += blockDim.x) {
     const int i = q % NB, j = (q / NB) % NB, k = NDIM == 3 ? q / (NB * NB) : 0;
     const int r = ((NDIM == 3 ? k + 1 : 0) * R + j + 1) * R + i + 1;
     const int c = ((NDIM == 3 ? k + NG : 0) * NP + j + NG) * NP + i + NG;
     const int ic[3] = {i, j, k};
-    auto bmean = [&](int j2, int d, int side) -> T {
-      const int cl = side ? c : c - po[d], cr = cl + po[d];
-      return T(0.5) * (ub[(size_t)(BX + j2) * S + cl] + ub[(size_t)(BX + j2) * S + cr]);
+    auto faces = [&](int d) {
+      CondFaces<T> f;
+      if (L.mode != 1) cond_faces<T>(ub + (size_t)BX * S, S, c, po[d], f);
+      return f;
     };
     auto face = [&](int d, const T* F) {
       if (R0) {
@@ -902,74 +956,123 @@ __global__ void __launch_bounds__(256) conduction_kernel(CondLaunch L) {
         if (ic[d] == NB - 1) R0[(size_t)(2 * d + 1) * NV * NB2 + (size_t)EN * NB2 + t1 * NB + t0] = -F[1];
       }
     };
-    const T acc = cond_rate<T, NDIM>(sT, sK, r, ro, gg, gmax, L.mode, bmean, face);
-    ub[(size_t)EN * S + c] = ub[(size_t)EN * S + c] + h * acc;
+    const T acc = cond_rate<T, NDIM>(sT, sK, r, ro, X, gmax, L.mode, faces, face);
+    ub[(size_t)EN * S + c] = ub[(size_t)EN * S + c] + pmul(h, acc);
   }
 }
 
-// Grid-wide barrier number k of a cooperative launch (the barrier words zeroed before it):
-// thread 0 of each CTA arrives on bar[0]; the last arrival resets it and opens the barrier by
-// storing k + 1 in bar[1]; the others wait for that value, giving up after ~2^31 clock cycles
-// (about a second).  Returns false when this CTA gave up (give_up: the test hook, at once).
-// Ordering: the CTA barrier orders the CTA's stores before thread 0's device-scope fence and
-// release (cumulative), and thread 0's acquire before the CTA's later loads; only thread 0
-// fences.
-__device__ __forceinline__ bool grid_barrier_bounded(unsigned* bar, unsigned nblocks, unsigned k, int give_up) {
-  __shared__ int ok_s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    int ok = 1;
-    if (give_up) {
-      ok = 0;
-    } else {
-      const unsigned arrived = atomicAdd(&bar[0], 1u) + 1u;
-      if (arrived == nblocks) {
-        atomicExch(&bar[0], 0u);
-        __threadfence();
-        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(bar + 1), "r"(k + 1u) : "memory");
-      } else {
-        const long long t0 = clock64();
-        for (;;) {
-          unsigned g;
-          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(g) : "l"(bar + 1) : "memory");
-          if (g == k + 1u) break;
-          if (clock64() - t0 > (1ll << 31)) { ok = 0; break; }
-        }
-      }
+// Exchange words of the conduction loop: a value with the number of the substep that made it,
+// in one 64-bit word (two for FP64), so the reader that finds the number it waits for has the
+// value with it -- no fence, flag or barrier between the two.
+__device__ __forceinline__ void put_word(unsigned long long* p, unsigned tag, unsigned bits) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(((unsigned long long)tag << 32) | bits) : "memory");
+}
+// waits for tag in *p (giving up after ~2^31 clock cycles, about a second, or at once for the
+// test hook)
+__device__ __forceinline__ bool get_word(const unsigned long long* p, unsigned tag, int give_up, unsigned& bits) {
+  if (give_up) return false;
+  const long long t0 = clock64();
+  for (;;) {
+    unsigned long long x;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(p) : "memory");
+    if ((unsigned)(x >> 32) == tag) {
+      bits = (unsigned)x;
+      return true;
     }
-    __threadfence();
-    ok_s = ok;
+    if (clock64() - t0 > (1ll << 31)) return false;
   }
-  __syncthreads();
-  return ok_s != 0;
+}
+template <typename T>
+struct XWords { static constexpr int N = sizeof(T) / 4; };
+__device__ __forceinline__ void put_value(unsigned long long* p, unsigned tag, float x) {
+  put_word(p, tag, __float_as_uint(x));
+}
+__device__ __forceinline__ void put_value(unsigned long long* p, unsigned tag, double x) {
+  put_word(p, tag, (unsigned)__double2loint(x));
+  put_word(p + 1, tag, (unsigned)__double2hiint(x));
+}
+__device__ __forceinline__ bool get_value(const unsigned long long* p, unsigned tag, int give_up, float& x) {
+  unsigned b = 0;
+  const bool ok = get_word(p, tag, give_up, b);
+  x = __uint_as_float(b);
+  return ok;
+}
+__device__ __forceinline__ bool get_value(const unsigned long long* p, unsigned tag, int give_up, double& x) {
+  unsigned lo = 0, hi = 0;
+  const bool ok = get_word(p, tag, give_up, lo) && get_word(p + 1, tag, give_up, hi);
+  x = __hiloint2double((int)hi, (int)lo);
+  return ok;
 }
 
-// The substep loop of cond_loop (CondLoopLaunch), one leaf per CTA of a cooperative launch.
-// The leaf's ring region (interior and one ghost layer) of every variable but psi stays in
-// shared memory over the loop.  Per substep: T and kappa on the ring, the interior energy
-// update (cond_rate, as conduction_kernel), the new interior energy into e_pp[it & 1], the
-// grid barrier, then the ring's ghost energy from the leaves it copies (all regions are
-// copies here, whose first ghost layer reads interior cells).  Leaves of problems with fewer
-// substeps take part in the barriers only.  After the loop the interior energy goes back to u;
-// its ghosts are stale, as after the per-substep path.  512 threads: a 16^2 leaf's ring region
-// (324 cells) and interior take one pass each (256 threads: 7.0 us per substep, 512: 6.6).
+// Shape of the loop's CTA: one thread per interior cell and one per ring cell of the leaf
+// (3D 8^3: the same threads take a cell of each kind).
+template <int NDIM, int NB>
+struct CondLoopShape {
+  static constexpr int R = NB + 2;
+  static constexpr int NR = NDIM == 3 ? R * R * R : R * R;
+  static constexpr int NI = NDIM == 3 ? NB * NB * NB : NB * NB;
+  static constexpr int NG1 = NR - NI;                          // ghost cells of the ring region
+  static constexpr int RING0 = NI + NG1 <= 512 ? NI : 0;       // first thread with a ring cell
+  static constexpr int THREADS = ((RING0 + NG1 > NI ? RING0 + NG1 : NI) + 31) / 32 * 32;
+  // every leaf's CTA has to be resident: in FP32 the registers are held to three 2D 16^2 or two
+  // 3D 8^3 leaves per SM (456 and 304 leaves on 152 SMs)
+  static constexpr int MIN_CTAS = NB == 8 ? (NDIM == 3 ? 2 : 6) : 3;
+  // the faces' mean field: 2D in registers over the loop; 3D (24 of them) from B in shared memory
+  static constexpr bool FACES_KEPT = NDIM == 2;
+  // k-th ghost cell of the ring region -> region coordinates
+  static __device__ __forceinline__ void ghost(int k, int& ri, int& rj, int& rk) {
+    rk = NDIM == 3 ? 0 : 1;
+    if (NDIM == 3) {
+      constexpr int PER = R * R - NB * NB;                      // ghosts of an inner plane
+      if (k < 2 * R * R) {
+        rk = k < R * R ? 0 : R - 1;
+        k %= R * R;
+        rj = k / R;
+        ri = k % R;
+        return;
+      }
+      k -= 2 * R * R;
+      rk = 1 + k / PER;
+      k %= PER;
+    }
+    if (k < 2 * R) {
+      rj = k < R ? 0 : R - 1;
+      ri = k % R;
+    } else {
+      k -= 2 * R;
+      rj = 1 + k / 2;
+      ri = k % 2 ? R - 1 : 0;
+    }
+  }
+};
+
+// The substep loop of one step (CondLoopLaunch), one leaf per CTA of a cooperative launch.
+// A thread keeps its cell's state -- an interior cell's, a ring cell's -- in registers over
+// the loop; T and kappa of the region are in shared memory.  Per substep: the interior
+// energies (cond_rate, as conduction_kernel), their new T and kappa, and, of the cells next to
+// the leaf's faces, the energy as an exchange word; each ring thread waits for the word of the
+// interior cell its ghost copies (all regions are copies here, whose first ghost layer reads
+// interior cells) and takes T and kappa of it.  Words alternate between two slots: a leaf
+// writes slot it & 1 again only after its neighbours' words of the substep between, which they
+// write after they have read that slot.  Leaves of different problems never wait for one
+// another, so each runs its own problem's substeps.
+//
+// A substep is latency: two CTA barriers and one trip of a word through L2.  256^2 (256 leaves
+// of 16^2, FP32): 6.4 us per substep with a grid barrier and the energies in the spare state
+// buffers -> 1.8 us.
 template <typename T, int NDIM, int NB>
-__global__ void __launch_bounds__(512) cond_loop_kernel(CondLoopLaunch L) {
+__global__ void __launch_bounds__(CondLoopShape<NDIM, NB>::THREADS, sizeof(T) == 4 ? CondLoopShape<NDIM, NB>::MIN_CTAS : 1)
+cond_loop_kernel(CondLoopLaunch L) {
   using G = Geo<NDIM, NB>;
-  constexpr int NP = G::NP, S = G::S;
-  constexpr int R = NB + 2;
-  constexpr int NR = NDIM == 3 ? R * R * R : R * R;
-  constexpr int NI = NDIM == 3 ? NB * NB * NB : NB * NB;
-  constexpr int NW = NV - 1;                        // rho, m, B, e (psi enters no T)
+  using SH = CondLoopShape<NDIM, NB>;
+  constexpr int NP = G::NP, S = G::S, R = SH::R, NR = SH::NR, NI = SH::NI, W = XWords<T>::N;
   extern __shared__ __align__(16) unsigned char csm[];
-  T* sW = reinterpret_cast<T*>(csm);                // [NW][NR]
-  T* sT = sW + (size_t)NW * NR;
+  T* sT = reinterpret_cast<T*>(csm);
   T* sK = sT + NR;
-  __shared__ GhostRegion reg[27];
-  const int blk = L.blocks[blockIdx.x];
+  T* sB = sK + NR;                                    // 3D: [3][NR]
+  __shared__ int failed;
+  const int blk = L.blocks[blockIdx.x], tid = threadIdx.x;
   const BlockGeo gg = L.geo[blk];
-  for (int q = threadIdx.x; q < 27; q += blockDim.x) reg[q] = L.regions[(size_t)blk * 27 + q];
   const int ns = L.nsub[gg.problem];
   const T h = (T)L.hsub[gg.problem];
   T* ub = (T*)L.u + (size_t)blk * NV * S;
@@ -979,78 +1082,93 @@ __global__ void __launch_bounds__(512) cond_loop_kernel(CondLoopLaunch L) {
   P.ch = T(0);
   P.tau = (T)L.tau;
   const T k0 = (T)L.kappa0, gmax = (T)L.grad_t_max;
-  auto padded = [&](int r) {                        // ring cell -> padded cell
-    const int ri = r % R, rj = (r / R) % R, rk = NDIM == 3 ? r / (R * R) : 0;
-    return ((NDIM == 3 ? rk + 1 : 0) * NP + rj + 1) * NP + ri + 1;
-  };
-  for (int r = threadIdx.x; r < NR; r += blockDim.x) {
-    const int c = padded(r);
-#pragma unroll
-    for (int v = 0; v < NW; ++v) sW[(size_t)v * NR + r] = ub[(size_t)v * S + c];
-  }
+  const CondDx<T> X(gg);
   const int ro[3] = {1, R, R * R};
-  unsigned fail = 0;
-  for (int it = 0; it < L.nmax; ++it) {
-    __syncthreads();
-    const bool active = it < ns;
-    if (active) {
-      for (int r = threadIdx.x; r < NR; r += blockDim.x) {
-        T w[NV];
+  const int po[3] = {1, NP, NP * NP};
+  unsigned long long* const slot[2] = {L.words, L.words + (size_t)L.nblocks * NI * W};
+  if (tid == 0) failed = 0;
+
+  // the interior cell
+  const bool inner = tid < NI;
+  int r = 0, c = 0;
+  bool shown = false;                                 // its energy is read by other leaves
+  T w[NV];
+  CondFaces<T> cf[SH::FACES_KEPT ? NDIM : 1];
+  if (inner) {
+    const int i = tid % NB, j = (tid / NB) % NB, k = NDIM == 3 ? tid / (NB * NB) : 0;
+    r = ((NDIM == 3 ? k + 1 : 0) * R + j + 1) * R + i + 1;
+    c = ((NDIM == 3 ? k + NG : 0) * NP + j + NG) * NP + i + NG;
+    shown = i == 0 || i == NB - 1 || j == 0 || j == NB - 1 || (NDIM == 3 && (k == 0 || k == NB - 1));
+    load_global<T>(ub, S, c, w);
+    if (SH::FACES_KEPT && L.mode != 1) {
 #pragma unroll
-        for (int v = 0; v < NW; ++v) w[v] = sW[(size_t)v * NR + r];
-        w[PSI] = T(0);
-        cond_tk<T>(w, P, k0, sT[r], sK[r]);
-      }
-      __syncthreads();
-      T* eb = (T*)L.e_pp[it & 1] + (size_t)blk * NV * S + (size_t)EN * S;
-      for (int q = threadIdx.x; q < NI; q += blockDim.x) {
-        const int i = q % NB, j = (q / NB) % NB, k = NDIM == 3 ? q / (NB * NB) : 0;
-        const int r = ((NDIM == 3 ? k + 1 : 0) * R + j + 1) * R + i + 1;
-        auto bmean = [&](int j2, int d, int side) -> T {
-          const int rl = side ? r : r - ro[d], rr = rl + ro[d];
-          return T(0.5) * (sW[(size_t)(BX + j2) * NR + rl] + sW[(size_t)(BX + j2) * NR + rr]);
-        };
-        auto face = [](int, const T*) {};
-        const T acc = cond_rate<T, NDIM>(sT, sK, r, ro, gg, gmax, L.mode, bmean, face);
-        // only this thread reads or writes cell r's energy in this phase (the rates read T,
-        // kappa and B)
-        const T en = sW[(size_t)EN * NR + r] + h * acc;
-        sW[(size_t)EN * NR + r] = en;
-        eb[padded(r)] = en;
-      }
+      for (int d = 0; d < NDIM; ++d) cond_faces<T>(ub + (size_t)BX * S, S, c, po[d], cf[SH::FACES_KEPT ? d : 0]);
     }
-    if (!grid_barrier_bounded(L.bar, (unsigned)L.nblocks, (unsigned)it, L.fail_waits)) {
-      fail = 4u;
+    cond_tk<T>(w, P, k0, sT[r], sK[r]);
+  }
+  auto keep_b = [&](int at, const T* q) {
+    if (!SH::FACES_KEPT)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) sB[j * NR + at] = q[BX + j];
+  };
+  if (inner) keep_b(r, w);
+  // the ring cell, and the word of the interior cell it copies
+  const bool ring = tid >= SH::RING0 && tid < SH::RING0 + SH::NG1;
+  int rg = 0;
+  size_t src = 0;
+  constexpr bool ONE_CELL = SH::RING0 == NI;          // no thread has a cell of each kind
+  T w2[ONE_CELL ? 1 : NV];
+  T* const wg = ONE_CELL ? w : w2;
+  if (ring) {
+    int ri, rj, rk;
+    SH::ghost(tid - SH::RING0, ri, rj, rk);
+    rg = ((NDIM == 3 ? rk : 0) * R + rj) * R + ri;
+    load_global<T>(ub, S, ((NDIM == 3 ? rk + 1 : 0) * NP + rj + 1) * NP + ri + 1, wg);
+    cond_tk<T>(wg, P, k0, sT[rg], sK[rg]);
+    keep_b(rg, wg);
+    const int rx = ri == 0 ? 0 : (ri == R - 1 ? 2 : 1), ry = rj == 0 ? 0 : (rj == R - 1 ? 2 : 1);
+    const int rz = NDIM == 3 ? (rk == 0 ? 0 : (rk == R - 1 ? 2 : 1)) : 1;
+    const GhostRegion g = L.regions[(size_t)blk * 27 + rx + 3 * ry + 9 * rz];
+    const int si = g.m[0] * (ri + 1) + g.a[0] - NG, sj = g.m[1] * (rj + 1) + g.a[1] - NG;
+    const int sk = NDIM == 3 ? g.m[2] * (rk + 1) + g.a[2] - NG : 0;
+    src = ((size_t)g.src * NI + (sk * NB + sj) * NB + si) * W;
+  }
+  const size_t own = ((size_t)blk * NI + tid) * W;
+  __syncthreads();
+  bool ok = true;
+  for (int it = 0; it < ns; ++it) {
+    const unsigned tag = L.tag0 + (unsigned)it;
+    const bool more = it + 1 < ns;
+    if (inner) {
+      auto faces = [&](int d) {
+        if (SH::FACES_KEPT) return cf[SH::FACES_KEPT ? d : 0];
+        CondFaces<T> f;
+        if (L.mode != 1) cond_faces<T>(sB, NR, r, ro[d], f);
+        return f;
+      };
+      auto face = [](int, const T*) {};
+      const T acc = cond_rate<T, NDIM>(sT, sK, r, ro, X, gmax, L.mode, faces, face);
+      w[EN] = w[EN] + pmul(h, acc);
+      if (shown && more) put_value(slot[it & 1] + own, tag, w[EN]);
+    }
+    if (!more) break;
+    __syncthreads();                                  // every rate has read T and kappa
+    if (inner) cond_tk<T>(w, P, k0, sT[r], sK[r]);
+    if (ring) {
+      if (get_value(slot[it & 1] + src, tag, L.fail_waits, wg[EN])) cond_tk<T>(wg, P, k0, sT[rg], sK[rg]);
+      else failed = 1;
+    }
+    __syncthreads();
+    if (failed) {
+      ok = false;
       break;
     }
-    if (active && it + 1 < ns) {
-      // the ring's ghost energy: region (rx, ry, rz) maps padded index i to m i + a of its
-      // source leaf, an interior cell of that leaf for the first ghost layer
-      const T* ebase = (const T*)L.e_pp[it & 1];
-      for (int r = threadIdx.x; r < NR; r += blockDim.x) {
-        const int ri = r % R, rj = (r / R) % R, rk = NDIM == 3 ? r / (R * R) : 1;
-        const int rx = ri == 0 ? 0 : (ri == R - 1 ? 2 : 1), ry = rj == 0 ? 0 : (rj == R - 1 ? 2 : 1);
-        const int rz = NDIM == 3 ? (rk == 0 ? 0 : (rk == R - 1 ? 2 : 1)) : 1;
-        if (rx == 1 && ry == 1 && rz == 1) continue;
-        const GhostRegion& g = reg[rx + 3 * ry + 9 * rz];
-        const int si = g.m[0] * (ri + 1) + g.a[0], sj = g.m[1] * (rj + 1) + g.a[1];
-        const int sk = NDIM == 3 ? g.m[2] * (rk + 1) + g.a[2] : 0;
-        const size_t sc = (size_t)g.src * NV * S + (size_t)EN * S + ((size_t)sk * NP + sj) * NP + si;
-        sW[(size_t)EN * NR + r] = __ldcg(ebase + sc);
-      }
-    }
   }
-  __syncthreads();
-  if (fail) {
-    if (threadIdx.x == 0) atomicOr(L.err_word, fail);
+  if (!ok) {
+    if (tid == 0) atomicOr(L.err_word, 4u);
     return;
   }
-  if (ns > 0)
-    for (int q = threadIdx.x; q < NI; q += blockDim.x) {
-      const int i = q % NB, j = (q / NB) % NB, k = NDIM == 3 ? q / (NB * NB) : 0;
-      const int r = ((NDIM == 3 ? k + 1 : 0) * R + j + 1) * R + i + 1;
-      ub[(size_t)EN * S + padded(r)] = sW[(size_t)EN * NR + r];
-    }
+  if (ns > 0 && inner) ub[(size_t)EN * S + c] = w[EN];
 }
 
 }  // namespace mapgb

@@ -91,10 +91,13 @@ struct map_pool {
   int nsm = 0;                 // SM count of the pool's device
   int fail_waits = 0;        // test hook: 1 every bounded wait gives up at once, 2 only the conduction loop's
   // conduction substep loop in one cooperative launch (map_set_conduction_loop): the switch,
-  // the grid barrier words, the CTAs that can be resident at once (-1: not asked yet) and
-  // whether every ghost region of the tree is a copy (-1: not checked for this tree)
+  // the exchange words (kept, grown to the largest tree that used them) with the last tag
+  // given out, the CTAs that can be resident at once (-1: not asked yet) and whether every
+  // ghost region of the tree is a copy (-1: not checked for this tree)
   int cond_loop = 1;
-  unsigned* gbar = nullptr;
+  unsigned long long* cond_words = nullptr;
+  size_t cond_words_n = 0;
+  unsigned cond_tag = 0;
   int cond_cap = -1;
   int cond_copies = -1;
   long long launches = 0;
@@ -242,8 +245,7 @@ int map_create_pool(const map_pool_desc* d, void* stream, map_pool** out) {
       cudaMalloc(&pool->err_word, sizeof(unsigned)) != cudaSuccess ||
       cudaMalloc(&pool->sums, sizeof(double) * kNV * pool->nprob) != cudaSuccess ||
       cudaMalloc(&pool->hsub, sizeof(double) * pool->nprob) != cudaSuccess ||
-      cudaMalloc(&pool->nsub, sizeof(int) * pool->nprob) != cudaSuccess ||
-      cudaMalloc(&pool->gbar, 2 * sizeof(unsigned)) != cudaSuccess)
+      cudaMalloc(&pool->nsub, sizeof(int) * pool->nprob) != cudaSuccess)
     return cleanup(MAP_ENOMEM, "cudaMalloc of the step constants failed");
   cudaMemsetAsync(pool->dyn, 0, sizeof(ProbDyn) * pool->nprob, pool->stream);
   cudaMemsetAsync(pool->err_word, 0, sizeof(unsigned), pool->stream);
@@ -262,7 +264,7 @@ int map_destroy_pool(map_pool* pool) {
   cudaFree(pool->dyn);
   cudaFree(pool->hsub);
   cudaFree(pool->nsub);
-  cudaFree(pool->gbar);
+  cudaFree(pool->cond_words);
   cudaFree(pool->err_word);
   cudaFree(pool->sums);
   cudaFree(pool->staging);
@@ -887,7 +889,22 @@ static bool cond_loop_usable(map_pool* pool, bool rf) {
     }
     pool->cond_copies = ok;
   }
-  return pool->cond_copies == 1;
+  if (pool->cond_copies != 1) return false;
+  // the exchange words; without the memory for them the per-substep path runs
+  const size_t words = (size_t)2 * pool->tree.nleaves * (interior_elems(pool) / kNV) * (pool->elem / 4);
+  if (words <= pool->cond_words_n && pool->cond_tag <= 0x7fffffffu) return true;
+  if (words > pool->cond_words_n) {
+    cudaFree(pool->cond_words);
+    pool->cond_words = nullptr;
+    pool->cond_words_n = 0;
+    if (cudaMalloc(&pool->cond_words, words * sizeof(unsigned long long)) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    pool->cond_words_n = words;
+  }
+  pool->cond_tag = 0;
+  return cudaMemsetAsync(pool->cond_words, 0, pool->cond_words_n * sizeof(unsigned long long), pool->stream) == cudaSuccess;
 }
 
 static int conduction_launches(map_pool* pool, const map_params* p) {
@@ -914,11 +931,11 @@ static int conduction_launches(map_pool* pool, const map_params* p) {
     // the per-substep path does), then every substep on the ring regions kept on chip
     int rc = fill_on(pool, pool->cur);
     if (rc) return rc;
-    CK(cudaMemsetAsync(pool->gbar, 0, 2 * sizeof(unsigned), pool->stream));
     CondLoopLaunch C;
     C.u = pool->buf[pool->cur];
-    C.e_pp[0] = pool->buf[1 - pool->cur];
-    C.e_pp[1] = pool->buf[2];
+    C.words = pool->cond_words;
+    C.tag0 = pool->cond_tag + 1;
+    pool->cond_tag += (unsigned)nmax;
     C.blocks = pool->dt.all_leaves;
     C.nblocks = pool->tree.nleaves;
     C.geo = pool->dt.geo;
@@ -930,8 +947,6 @@ static int conduction_launches(map_pool* pool, const map_params* p) {
     C.mode = p->conduction;
     C.hsub = pool->hsub;
     C.nsub = pool->nsub;
-    C.nmax = nmax;
-    C.bar = pool->gbar;
     C.err_word = pool->err_word;
     C.fail_waits = pool->fail_waits != 0;
     if (DISPATCH(pool, cond_loop, C) == cudaSuccess) {

@@ -241,13 +241,12 @@ cudaError_t launch_conduction_T(const KernelConfig& kc, const CondLaunch& L, cud
 #undef CALL_COND
 }
 
-// the conduction loop (cond_loop_kernel): the ring region of every variable but psi, T and
-// kappa in shared memory; 3D 16^3 leaves would need 233 KB and are left to the per-substep
-// kernels
+// the conduction loop (cond_loop_kernel): T and kappa (3D: and B) of the ring region in shared
+// memory, one thread per cell; 3D 16^3 leaves have more cells than a CTA has threads and are left to the
+// per-substep kernels
 template <typename T, int NDIM, int NB>
 constexpr size_t cond_loop_smem() {
-  constexpr int R = NB + 2;
-  return (size_t)(NV + 1) * (NDIM == 3 ? R * R * R : R * R) * sizeof(T);
+  return (size_t)(CondLoopShape<NDIM, NB>::FACES_KEPT ? 2 : 5) * CondLoopShape<NDIM, NB>::NR * sizeof(T);
 }
 
 template <typename T, int NDIM, int NB>
@@ -263,7 +262,8 @@ int cond_loop_capacity_one(int nsm) {
       return 0;
     }
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 512, smem) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, CondLoopShape<NDIM, NB>::THREADS, smem) !=
+        cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
@@ -280,8 +280,8 @@ cudaError_t launch_cond_loop_one(const CondLoopLaunch& L, cudaStream_t s) {
   } else {
     CondLoopLaunch A = L;
     void* args[] = {&A};
-    return cudaLaunchCooperativeKernel((const void*)cond_loop_kernel<T, NDIM, NB>, dim3(L.nblocks), dim3(512), args,
-                                       cond_loop_smem<T, NDIM, NB>(), s);
+    return cudaLaunchCooperativeKernel((const void*)cond_loop_kernel<T, NDIM, NB>, dim3(L.nblocks),
+                                       dim3(CondLoopShape<NDIM, NB>::THREADS), args, cond_loop_smem<T, NDIM, NB>(), s);
   }
 }
 

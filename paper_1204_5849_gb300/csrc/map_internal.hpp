@@ -221,12 +221,13 @@ struct CondLaunch {
 };
 
 // The whole conduction substep loop of one step in one cooperative launch (single-level
-// meshes whose ghost regions are all copies): each CTA keeps its leaf's ring region in
-// shared memory and exchanges the energy of its interior through e_pp[it & 1] (the energy
-// slices of two spare state buffers), one bounded grid barrier per substep.
+// meshes whose ghost regions are all copies): each CTA keeps its leaf on chip and exchanges
+// the energies next to its faces with the leaves it borders through words[2][leaf][cell], each
+// word carrying the substep's tag.
 struct CondLoopLaunch {
   void* u;                 // the state: the ring region is read, the interior energy written
-  void* e_pp[2];           // two state buffers whose energy slices carry the exchange
+  unsigned long long* words;   // 2 slots of nblocks x nb^ndim values (one word each, two in FP64)
+  unsigned tag0;           // tag of the first substep; no earlier launch used it or a later one
   const int* blocks;       // leaves, one CTA each
   int nblocks;
   const BlockGeo* geo;
@@ -235,10 +236,8 @@ struct CondLoopLaunch {
   int mode;                // 1 isotropic, 2 along B
   const double* hsub;
   const int* nsub;
-  int nmax;                // substeps of the problem with the most
-  unsigned* bar;           // grid barrier words (zeroed before the launch)
   unsigned* err_word;
-  int fail_waits;          // test hook: the barrier gives up at once
+  int fail_waits;          // test hook: the waits give up at once
 };
 
 struct FillLaunch {
