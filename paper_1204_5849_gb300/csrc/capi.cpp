@@ -730,11 +730,11 @@ int map_cfl_dt(map_pool* pool, const map_params* p, double* dt_out) {
 }
 
 // Grid of the FP32 single step launch: the tuned one, else one CTA per block in 3D and, in
-// 2D (256-cell blocks, whose per-block reductions weigh), a persistent grid of four CTAs per
-// SM (the residency of the 128-thread 2D FP32 kernels).
-static int step_grid(const map_pool* pool) {
+// 2D (256-cell blocks, whose per-block reductions weigh), a persistent grid of as many CTAs
+// per SM as the 128-thread 2D FP32 kernels have resident: three for MMC, else four.
+static int step_grid(const map_pool* pool, const map_params* p) {
   if (pool->tune_grid > 0) return pool->tune_grid;
-  if (!is64(pool) && pool->ndim == 2 && pool->nsm > 0) return 4 * pool->nsm;
+  if (!is64(pool) && pool->ndim == 2 && pool->nsm > 0) return (p->scheme == MAP_MMC && pool->nb == 16 ? 3 : 4) * pool->nsm;
   return 0;
 }
 
@@ -818,7 +818,7 @@ static int step_launches(map_pool* pool, const map_params* p, bool fused) {
       }
     } else {
       S.nblocks = pool->partial ? D.n_act : t.nleaves;
-      S.grid = step_grid(pool);
+      S.grid = step_grid(pool, p);
       const int rcl = step_block_list(pool, S.grid, &S.blocks);
       if (rcl) return rcl;
       if (S.nblocks > 0) CK(DISPATCH(pool, step, S));
@@ -1382,7 +1382,7 @@ int map_autotune(map_pool* pool, const map_params* p, int reps, map_tune_result*
   int bg = 0, bwp = dwp, bwf = dwf;
   rc = trial(0, dwp, dwf, &best);
   const float base = best;
-  if (rc == MAP_OK && step_grid(pool) > 0) {
+  if (rc == MAP_OK && step_grid(pool, p) > 0) {
     // the default is persistent here: try one CTA per block as well
     rc = trial(pool->tree.nleaves, dwp, dwf, &t);
     if (rc == MAP_OK && t < best) { best = t; bg = pool->tree.nleaves; }

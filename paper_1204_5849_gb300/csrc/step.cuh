@@ -26,6 +26,7 @@
 
 #include "chain.cuh"
 #include "map_internal.hpp"
+#include "mmc2d.cuh"
 #include "physics.cuh"
 
 namespace mapgb {
@@ -80,6 +81,10 @@ struct Geo {
   static constexpr int NFACE = NB * (NB + 1);
 };
 
+// 2D MMC runs the phases of mmc2d.cuh, with the kept fluxes of u in shared memory.
+template <int NDIM, int SCHEME>
+struct Mmc2d { static constexpr bool value = NDIM == 2 && SCHEME == SCH_MMC; };
+
 template <typename T, int NDIM, int NB, int SCHEME>
 __host__ __device__ constexpr size_t step_smem_bytes(bool resistive) {
   using G = Geo<NDIM, NB>;
@@ -89,6 +94,7 @@ __host__ __device__ constexpr size_t step_smem_bytes(bool resistive) {
   if (nf < (size_t)(NV + 1) * 32 * 2) nf = (size_t)(NV + 1) * 32 * 2;  // reused for reductions
   n += nf;
   if (resistive) n += (size_t)G::WPL * 3 * G::RING;                 // J window (ring)
+  if (Mmc2d<NDIM, SCHEME>::value) n += (size_t)2 * mmc2d::NQ * G::P2;   // kept fluxes of u
   return 256 + n * sizeof(T);                                       // 256 B: mbarriers, block constants
 }
 
@@ -456,14 +462,16 @@ __device__ __forceinline__ void two_sum_acc(T& hi, T& lo, T h2, T l2) {
 // Resident CTAs per SM the register budget is sized for: the 3D 8^3 window (at most 36 KB of
 // shared memory) lets 6 CTAs reside, so asking for 8 would only cap the registers at 128 and
 // spill the column state; four 128-thread 2D 16^2 CTAs take the 128 registers two 256-thread
-// ones did.
-template <typename T, int NDIM, int NB>
+// ones did.  2D MMC's kept fluxes (68 KB of shared memory for 16^2) let three reside, whose
+// face walk then has 168 registers.
+template <typename T, int NDIM, int NB, int SCHEME>
 constexpr int step_min_ctas() {
-  return sizeof(T) != 4 ? 1 : NB == 16 ? (NDIM == 2 ? 4 : 2) : NDIM == 3 ? 6 : 8;
+  return sizeof(T) != 4 ? 1 : NB == 16 ? (NDIM == 2 ? (Mmc2d<NDIM, SCHEME>::value ? 3 : 4) : 2)
+                                       : NDIM == 3 ? 6 : (Mmc2d<NDIM, SCHEME>::value ? 6 : 8);
 }
 
 template <typename T, int NDIM, int NB, int SCHEME, int LIM, int STAGE, int FLX, bool RFX>
-__global__ void __launch_bounds__(step_threads<T, NDIM, NB>(), step_min_ctas<T, NDIM, NB>())
+__global__ void __launch_bounds__(step_threads<T, NDIM, NB>(), step_min_ctas<T, NDIM, NB, SCHEME>())
 step_kernel(StepArgsT<T> A) {
   using G = Geo<NDIM, NB>;
   constexpr int NP = G::NP, P2 = G::P2, NZ = G::NZ, S = G::S;
@@ -483,6 +491,7 @@ step_kernel(StepArgsT<T> A) {
   size_t nf = (size_t)2 * NV * NFACE;
   if (nf < (size_t)(NV + 1) * 32 * 2) nf = (size_t)(NV + 1) * 32 * 2;
   T* sj = sf + nf;
+  T* sr = sj + (A.resistive ? (size_t)WPL * 3 * RING : 0);            // 2D MMC: kept fluxes of u
   __shared__ PushEntry spush[27];
 
   const int tid = threadIdx.x;
@@ -597,7 +606,11 @@ step_kernel(StepArgsT<T> A) {
 #pragma unroll
         for (int v = 0; v < NV; ++v) acc[v] = w[v];
         T* tp = tslot(z);
-        if (SCHEME == SCH_MMC) {
+        if constexpr (Mmc2d<NDIM, SCHEME>::value) {
+          mmc2d::predict<T, NB>(ul[1], sr, c, lam, P, acc);
+#pragma unroll
+          for (int v = 0; v < NV; ++v) tp[v * RING + r] = acc[v];
+        } else if (SCHEME == SCH_MMC) {
           T wm[NV], wp[NV], hp[NV], hm[NV];
           ldw<T, P2>(ul[1], c - 1, wm);
           ldw<T, P2>(ul[1], c + 1, wp);
@@ -900,11 +913,19 @@ step_kernel(StepArgsT<T> A) {
         if (!ok) break;
         read_constants();
         if (PREF && tid == 0) kc[16] = total_pressure(uslot(0), cown);           // read after the next barrier
-        if (PRED) {
+        if constexpr (Mmc2d<NDIM, SCHEME>::value) {
+          mmc2d::cell_fluxes<T, NB, NT>(su, sr, P, tid);
+          __syncthreads();
           work(0, true, 0, false);
           __syncthreads();
+          mmc2d::faces<T, NB, NT, LIM>(su, sut, sr, sfx, sfy, P, tid);
+        } else {
+          if (PRED) {
+            work(0, true, 0, false);
+            __syncthreads();
+          }
+          work(0, false, 0, true);
         }
-        work(0, false, 0, true);
       }
       __syncthreads();
       // plane z-1's values for this plane's sources; plane z's are kept for the next, as the
