@@ -607,7 +607,8 @@ step_kernel(StepArgsT<T> A) {
         for (int v = 0; v < NV; ++v) acc[v] = w[v];
         T* tp = tslot(z);
         if constexpr (Mmc2d<NDIM, SCHEME>::value) {
-          mmc2d::predict<T, NB>(ul[1], sr, c, lam, P, acc);
+          if constexpr (sizeof(T) == 4) mmc2d::predict<NB>(ul[1], sr, c, lam, P, acc);
+          else mmc2d::predict<T, NB>(ul[1], sr, c, lam, P, acc);
 #pragma unroll
           for (int v = 0; v < NV; ++v) tp[v * RING + r] = acc[v];
         } else if (SCHEME == SCH_MMC) {
@@ -914,11 +915,13 @@ step_kernel(StepArgsT<T> A) {
         read_constants();
         if (PREF && tid == 0) kc[16] = total_pressure(uslot(0), cown);           // read after the next barrier
         if constexpr (Mmc2d<NDIM, SCHEME>::value) {
-          mmc2d::cell_fluxes<T, NB, NT>(su, sr, P, tid);
+          if constexpr (sizeof(T) == 4) mmc2d::cell_fluxes<NB, NT>(su, sr, P, tid);
+          else mmc2d::cell_fluxes<T, NB, NT>(su, sr, P, tid);
           __syncthreads();
           work(0, true, 0, false);
           __syncthreads();
-          mmc2d::faces<T, NB, NT, LIM>(su, sut, sr, sfx, sfy, P, tid);
+          if constexpr (sizeof(T) == 4) mmc2d::faces_f32<NB, NT, LIM>(su, sut, sr, sfx, sfy, P, tid);
+          else mmc2d::faces<T, NB, NT, LIM>(su, sut, sr, sfx, sfy, P, tid);
         } else {
           if (PRED) {
             work(0, true, 0, false);
