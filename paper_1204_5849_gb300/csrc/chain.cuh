@@ -21,6 +21,9 @@ namespace mapgb {
 
 __device__ __forceinline__ void chain_begin() { cudaGridDependencySynchronize(); }
 
+// Lets the next kernel of the chain be set up once every block has called this or ended.
+__device__ __forceinline__ void chain_release() { cudaTriggerProgrammaticLaunchCompletion(); }
+
 template <typename... P, typename... A>
 inline cudaError_t launch_chained(void (*kern)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args) {
   cudaLaunchConfig_t cfg{};

@@ -22,6 +22,7 @@ __global__ void __launch_bounds__(64) finalize_kernel(FinalizeLaunch L) {
   const int p = blockIdx.x, lane = threadIdx.x & 31;
   const bool dt_warp = threadIdx.x < 32;
   const double log_cd = !dt_warp && L.cp_mode == MAP_CP_FROM_CD ? log(L.c_d) : 0.0;
+  chain_release();
   chain_begin();
   const ProbDyn d = L.dyn[p];
   __syncthreads();                       // both warps hold the maxima before they are reset

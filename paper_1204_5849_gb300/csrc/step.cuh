@@ -515,6 +515,18 @@ step_kernel(StepArgsT<T> A) {
 #pragma unroll
       for (int k = 0; k < 16; ++k) sched[q][k] = A.sched[q][k];
   }
+  // 2D, whose blocks are short: a block's table entries, which no kernel of the chain writes, are
+  // read ahead -- the first block's before the wait for the kernels before this one, the next
+  // one's during each block -- and the constants written when problem or level change.  (3D
+  // keeps none of it over its planes: the registers cost the 16^3 kernel more.)
+  int bi = blockIdx.x, blk = 0, prob = 0, level = 0;
+  auto table = [&]() {
+    blk = A.blocks[bi];
+    prob = A.geo[blk].problem;
+    level = A.geo[blk].level;
+  };
+  if (NDIM == 2) table();
+  bool new_consts = true;               // kc has to be written (3D: for every block)
   __syncthreads();
   chain_begin();
   unsigned phase = 0;                                   // parity bit per u slot
@@ -528,9 +540,8 @@ step_kernel(StepArgsT<T> A) {
   for (int v = 0; v < NV; ++v) { csum[v] = T(0); ccmp[v] = T(0); }
   unsigned errbits = 0;
 
-  for (int bi = blockIdx.x; bi < A.nblocks; bi += gridDim.x) {
-    const int blk = A.blocks[bi];
-    const BlockGeo gg = A.geo[blk];
+  for (;;) {
+    if (NDIM == 3) table();
     if (A.pushes && tid < 27) spush[tid] = A.pushes[(size_t)blk * 27 + tid];   // read after the first barrier
     if (RFX && tid == 0) srl = A.refl[blk];             // read after the first barrier
     const T* ub = A.u_in + (size_t)blk * NV * S;
@@ -860,6 +871,8 @@ step_kernel(StepArgsT<T> A) {
       }
     };
 
+    int blk_next = 0;
+    if (NDIM == 2 && bi + (int)gridDim.x < A.nblocks) blk_next = A.blocks[bi + gridDim.x];
     T Fzlo[NV], uprev[NV];
     // the own column's u~ B_z, psi and J of the previous plane (its ring slot is reused)
     T car_bz = T(0), car_psi = T(0), car_j[3] = {T(0), T(0), T(0)};
@@ -872,25 +885,31 @@ step_kernel(StepArgsT<T> A) {
         issue_plane(2);
         issue_plane(3);
       }
-      // per-block constants, rounded to T while the first planes are in flight.  dt/dx at
-      // level L is 2^L dt/dx0 exactly, and rounding to T commutes with scaling by powers of
-      // two, so these equal the FP64 dt/dx, (dt/2)/dx, 2 dx, dx, dt, dt/2 rounded to T
-      // without an FP64 division per block (the FP64 pipe runs at 1/64 of the FP32 rate)
-      const ProbDyn dy = A.dyn[gg.problem];
-      const T scale = (T)(1 << gg.level);
-      for (int d = 0; d < 3; ++d) {
-        const T lam_d = (T)dy.lam0[d] * (d < NDIM ? scale : T(1));
-        const T dx_d = (T)gg.dx[d];
-        kc[d] = lam_d;
-        kc[3 + d] = T(0.5) * lam_d;
-        kc[6 + d] = T(2) * dx_d;
-        kc[9 + d] = dx_d;
+    }
+    if (new_consts && tid < 9) {
+      // block constants, rounded to T while the first planes are in flight, one per lane of warp
+      // 0 (a conversion from FP64 at 1/64 of the FP32 rate costs a warp the same for one lane as
+      // for all; one thread converting all of them had held every block up by 2000 cycles).  dt/dx
+      // at level L is 2^L dt/dx0 exactly, and rounding to T commutes with scaling by powers of
+      // two, so these equal the FP64 dt/dx, (dt/2)/dx, 2 dx, dx, dt, dt/2 rounded to T without an
+      // FP64 division per block
+      const ProbDyn* dy = A.dyn + prob;
+      const double* src = tid < 3 ? &dy->lam0[tid] : tid < 6 ? &A.geo[blk].dx[tid - 3]
+                          : tid == 6 ? &dy->dt : tid == 7 ? &dy->damp : &dy->ch;
+      const T x = (T)*src;
+      if (tid < 3) {
+        const T lam_d = x * (tid < NDIM ? (T)(1 << level) : T(1));
+        kc[tid] = lam_d;
+        kc[3 + tid] = T(0.5) * lam_d;
+      } else if (tid < 6) {
+        kc[3 + tid] = T(2) * x;
+        kc[6 + tid] = x;
+      } else if (tid == 6) {
+        kc[12] = x;
+        kc[13] = T(0.5) * x;
+      } else {
+        kc[7 + tid] = x;                                // damping 14, c_h 15
       }
-      const T dt_T = (T)dy.dt;
-      kc[12] = dt_T;
-      kc[13] = T(0.5) * dt_T;
-      kc[14] = (T)dy.damp;
-      kc[15] = (T)dy.ch;
     }
     // 3D: iteration z predicts plane z+1 and updates plane z (z >= NG); one call site per
     // work-item kind keeps the kernel's code small.  2D: a single plane.
@@ -1128,16 +1147,20 @@ step_kernel(StepArgsT<T> A) {
       __syncthreads();
     }
     if (!ok) break;
+    const bool last = bi + (int)gridDim.x >= A.nblocks;
+    if (last) chain_release();
     // reductions of the fused diagnostics, in T within each warp (TwoSum pairs for the sums),
     // then FP64 across warps.  The per-thread maxima and compensated sums keep accumulating
     // over the CTA's consecutive blocks of one problem and level (equal cell volumes) and are
     // reduced once that run ends -- a persistent grid given contiguous block ranges reduces
     // once per run instead of once per block (the decision is the same on every thread)
-    bool flush = true;
-    if (bi + (int)gridDim.x < A.nblocks) {
-      const BlockGeo gn = A.geo[A.blocks[bi + gridDim.x]];
-      flush = gn.problem != gg.problem || gn.level != gg.level;
+    int prob_next = prob, level_next = level;
+    if (!last) {
+      if (NDIM == 3) blk_next = A.blocks[bi + gridDim.x];
+      prob_next = A.geo[blk_next].problem;
+      level_next = A.geo[blk_next].level;
     }
+    const bool flush = last || prob_next != prob || level_next != level;
     if ((A.dyn_next || A.sums) && flush) {
       double* red = reinterpret_cast<double*>(sf);     // (NV+1) x 32 doubles
       const int lane = tid & 31, wid = tid >> 5;
@@ -1146,20 +1169,44 @@ step_kernel(StepArgsT<T> A) {
         const T t = __shfl_xor_sync(0xffffffffu, am, o);
         am = (t != t || am != am) ? (T)NAN : dmax<T>(am, t);
       }
-      // after the butterflies every lane holds the warp's (hi, lo) of variable v; lane v
-      // keeps variable v's pair and widens it to one FP64 value (one conversion per warp:
-      // the FP64 pipe runs at 1/64 of the FP32 rate), lane NV the alpha maximum
-      T hsel = am, lsel = T(0);
+      // the warp's (hi, lo) of variable v end in lane v, which widens the pair to one FP64 value
+      // (one conversion per warp: the FP64 pipe runs at 1/64 of the FP32 rate); lane NV takes the
+      // alpha maximum
+      // (the first eight by halving: after the exchange over a lane bit a lane keeps the half of
+      // its variables whose index agrees with that bit, so lane v ends with variable v; 14 pair
+      // additions in place of 45)
+      static_assert(NV == 9, "eight variables halve over three lane bits, the ninth goes alone");
+      T hi[NV], lo[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        T hi = csum[v], lo = -ccmp[v];
-        for (int o = 16; o > 0; o >>= 1) {
-          const T h2 = __shfl_xor_sync(0xffffffffu, hi, o);
-          const T l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-          two_sum_acc<T>(hi, lo, h2, l2);
-        }
-        if (lane == v) { hsel = hi; lsel = lo; }
+        hi[v] = csum[v];
+        lo[v] = -ccmp[v];
       }
+#pragma unroll
+      for (int b = 4; b > 0; b >>= 1) {
+        const bool up = (lane & b) != 0;
+#pragma unroll
+        for (int v = 0; v < b; ++v) {
+          const T gh = up ? hi[v] : hi[v + b], gl = up ? lo[v] : lo[v + b];
+          hi[v] = up ? hi[v + b] : hi[v];
+          lo[v] = up ? lo[v + b] : lo[v];
+          const T h2 = __shfl_xor_sync(0xffffffffu, gh, b);
+          const T l2 = __shfl_xor_sync(0xffffffffu, gl, b);
+          two_sum_acc<T>(hi[v], lo[v], h2, l2);
+        }
+      }
+      for (int o = 8; o <= 16; o <<= 1) {
+        const T h2 = __shfl_xor_sync(0xffffffffu, hi[0], o);
+        const T l2 = __shfl_xor_sync(0xffffffffu, lo[0], o);
+        two_sum_acc<T>(hi[0], lo[0], h2, l2);
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        const T h2 = __shfl_xor_sync(0xffffffffu, hi[NV - 1], o);
+        const T l2 = __shfl_xor_sync(0xffffffffu, lo[NV - 1], o);
+        two_sum_acc<T>(hi[NV - 1], lo[NV - 1], h2, l2);
+      }
+      const T hsel = lane < NV - 1 ? hi[0] : (lane == NV ? am : hi[NV - 1]);
+      const T lsel = lane < NV - 1 ? lo[0] : lo[NV - 1];
       if (lane < NV) red[lane * 32 + wid] = (double)hsel + (double)lsel;
       if (lane == NV) red[NV * 32 + wid] = (double)hsel;
       __syncthreads();
@@ -1174,18 +1221,27 @@ step_kernel(StepArgsT<T> A) {
             a2 = (t != t || a2 != a2) ? __longlong_as_double(0x7ff8000000000000ll) : fmax(a2, t);
           }
           // alpha >= 0: its IEEE bit pattern orders like the value (NaN above everything)
-          if (A.dyn_next) atomicMax(&A.dyn_next[gg.problem].alpha_bits, (unsigned long long)__double_as_longlong(a2));
+          if (A.dyn_next) atomicMax(&A.dyn_next[prob].alpha_bits, (unsigned long long)__double_as_longlong(a2));
         } else if (A.sums) {
-          const double vol = gg.dx[0] * gg.dx[1] * (NDIM == 3 ? gg.dx[2] : 1.0);
+          const double* dx = A.geo[blk].dx;
+          const double vol = dx[0] * dx[1] * (NDIM == 3 ? dx[2] : 1.0);
           double t = 0.0;
           for (int q = 0; q < nw; ++q) t += red[tid * 32 + q];
-          atomicAdd(&A.sums[gg.problem * NV + tid], t * vol);
+          atomicAdd(&A.sums[prob * NV + tid], t * vol);
         }
       }
       __syncthreads();
       alpha_max = T(0);
 #pragma unroll
       for (int v = 0; v < NV; ++v) { csum[v] = T(0); ccmp[v] = T(0); }
+    }
+    if (last) break;
+    bi += gridDim.x;
+    if (NDIM == 2) {
+      new_consts = prob_next != prob || level_next != level;
+      blk = blk_next;
+      prob = prob_next;
+      level = level_next;
     }
   }
   if (*status != 0) {
