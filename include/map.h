@@ -191,8 +191,8 @@ int map_step(map_pool* pool, const map_params* p);
 /* nsteps x (ghost fill, dt on the device, step), asynchronous: the batched form.  The
  * step kernel also reduces alpha_g of the new state (the next dt) and the FP64
  * conservation sums of the new state, so a separate CFL pass runs only before the first
- * step after the state changed outside this call.  The step sequence is captured once per
- * starting buffer into a CUDA graph and replayed.  map_get_speeds reads the last dt. */
+ * step after the state changed outside this call.  The steps are plain launches on the
+ * pool's stream.  map_get_speeds reads the last dt. */
 int map_advance(map_pool* pool, const map_params* p, int nsteps);
 
 /* Device error word accumulated by the steps since the last check (rho <= 0, p < 0,

@@ -1,5 +1,5 @@
 // capi.cpp -- the extern "C" ABI declared in include/map.h: pool memory, tree tables,
-// the step sequence and its CUDA-graph replay.
+// the step sequence.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>
@@ -102,10 +102,6 @@ struct map_pool {
   int cond_copies = -1;
   long long launches = 0;
   std::string err;
-  // graph cache, one per starting buffer parity q and fill kind (2q + 1: residual fill)
-  cudaGraphExec_t graph[4] = {nullptr, nullptr, nullptr, nullptr};
-  long long graph_kernels[4] = {0, 0, 0, 0};
-  map_params graph_params{};
   // conduction substep loops captured as graphs, keyed by substep count, buffer, the pushed
   // state of the first fill and reflux (cond_params: the parameters they were captured for)
   struct CondGraph {
@@ -117,7 +113,6 @@ struct map_pool {
   CondGraph cond_graph[8];
   int cond_next = 0;
   map_params cond_params{};
-  bool graph_valid[4] = {false, false, false, false};
 };
 
 static std::string g_create_error;
@@ -172,11 +167,6 @@ static void drop_graphs(map_pool* pool) {
   for (auto& c : pool->cond_graph) {
     if (c.ex) cudaGraphExecDestroy(c.ex);
     c = map_pool::CondGraph();
-  }
-  for (int q = 0; q < 4; ++q) {
-    if (pool->graph[q]) cudaGraphExecDestroy(pool->graph[q]);
-    pool->graph[q] = nullptr;
-    pool->graph_valid[q] = false;
   }
 }
 
@@ -1115,53 +1105,20 @@ int map_advance(map_pool* pool, const map_params* p, int nsteps) {
     pool->sums_valid = false;
     return MAP_OK;
   }
-  if (!params_equal(pool->graph_params, *p)) {
-    drop_graphs(pool);
-    pool->graph_params = *p;
-  }
   if (!pool->alpha_ready) {
     rc = alpha_device(pool, p);
     if (rc) return rc;
     pool->alpha_ready = true;
   }
+  // Plain launches: a step is two of them on a uniform mesh, up to twenty on a refined one, and the host
+  // enqueues a launch in about 2.5 us, faster than the device runs it, while a step replayed as
+  // one CUDA graph left 4 to 5 us between two graphs, across which no launch overlapped the
+  // kernel before it.  Per pass, a graph per step -> this: 128^2 MMC, ten steps 218 -> 174 us;
+  // 720x528 HLLC, four steps 262 -> 250; 112x80x96 MMC 1004 -> 990; 2992-leaf rotor (17
+  // launches a step) 848 -> 844; 9472-leaf octree 4645 -> 4643.
   for (int s = 0; s < nsteps; ++s) {
-    const int q = pool->cur;
-    const int gi = 2 * q + (pool->pushed[q] ? 1 : 0);
-    if (!pool->graph_valid[gi]) {
-      // first step from this buffer: run eagerly (this also sets kernel attributes), then
-      // capture the same sequence starting from buffer q for later replays
-      rc = advance_once(pool, p);
-      if (rc) return rc;
-      const int after = pool->cur;
-      const long long before = pool->launches;
-      pool->cur = q;
-      cudaGraph_t g = nullptr;
-      if (cudaStreamBeginCapture(pool->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-        rc = advance_once(pool, p);
-        cudaError_t ce = cudaStreamEndCapture(pool->stream, &g);
-        if (rc == MAP_OK && ce == cudaSuccess && g) {
-          size_t nnodes = 0;
-          cudaGraphGetNodes(g, nullptr, &nnodes);
-          cudaGraphExec_t ex = nullptr;
-          if (cudaGraphInstantiate(&ex, g, 0) == cudaSuccess) {
-            pool->graph[gi] = ex;
-            pool->graph_valid[gi] = true;
-            pool->graph_kernels[gi] = pool->launches - before;
-            (void)nnodes;
-          }
-        }
-        if (g) cudaGraphDestroy(g);
-        cudaGetLastError();
-      }
-      pool->cur = after;
-      pool->launches = before;
-      if (rc) return rc;
-      continue;
-    }
-    CK(cudaGraphLaunch(pool->graph[gi], pool->stream));
-    pool->launches += pool->graph_kernels[gi];
-    pool->cur = 1 - q;
-    pool->pushed[1 - q] = true;
+    rc = advance_once(pool, p);
+    if (rc) return rc;
   }
   pool->have_dt = false;
   pool->sums_valid = true;
@@ -1281,7 +1238,7 @@ int map_adapt(map_pool* pool, const map_params* p, const map_refine_params* r, i
            plan[l].ijk[2] == pool->tree.blk_ijk[3 * id + 2];
   }
   *n_out = (int)plan.size();
-  if (same) return MAP_OK;                       // nothing to do: tree, tables and graphs stay
+  if (same) return MAP_OK;                       // nothing to do: tree and tables stay
   return map_regrid(pool, plan.data(), (int)plan.size());
 }
 
