@@ -35,7 +35,9 @@ __device__ __forceinline__ T dmax(T a, T b) { return a > b ? a : b; }
 // a / b.  FP64: the plain quotient (rounds as the same formula written in plain C).  FP32:
 // the fast quotient, reciprocal times numerator (within 2 ulp); every FP32 quotient on the
 // step path has a denominator (a density, a cell spacing, a sum of slopes, a WENO weight sum)
-// far below the 2^126 range where the fast form flushes to zero.
+// far below the 2^126 range where the fast form flushes to zero.  (HLLC and HLLD, a dozen
+// quotients a face: with the full-range quotient of a plain a / b four steps of a 720x528 mesh
+// took 161.5 us in place of 157.7.)
 template <typename T>
 __device__ __forceinline__ T qdiv(T a, T b) { return a / b; }
 template <>
@@ -172,7 +174,7 @@ __device__ __forceinline__ T fast_speed(const T* w, T p, const Phys<T>& P) {
 template <typename T, int D>
 __device__ __forceinline__ void hllc_flux(const T* a, const T* b, const Phys<T>& P, T* f) {
   const T ch = P.ch;
-  const T bm = ch > T(0) ? T(0.5) * (a[BX + D] + b[BX + D]) - (b[PSI] - a[PSI]) / (T(2) * ch)
+  const T bm = ch > T(0) ? T(0.5) * (a[BX + D] + b[BX + D]) - qdiv<T>(b[PSI] - a[PSI], T(2) * ch)
                          : T(0.5) * (a[BX + D] + b[BX + D]);
   T w[2][NV], F[2][NV], u[2], cf[2], pt[2];
 #pragma unroll
@@ -185,7 +187,7 @@ __device__ __forceinline__ void hllc_flux(const T* a, const T* b, const Phys<T>&
     w[k][EN] = q[EN] + T(0.5) * (bm * bm - q[BX + D] * q[BX + D]);
     const T pw = pressure<T>(w[k], P);
     flux_p<T, D>(w[k], pw, P, F[k]);
-    u[k] = w[k][MX + D] / w[k][RHO];
+    u[k] = qdiv<T>(w[k][MX + D], w[k][RHO]);
     cf[k] = fast_speed<T, D>(w[k], pw, P);
     pt[k] = p + T(0.5) * (w[k][BX] * w[k][BX] + w[k][BY] * w[k][BY] + w[k][BZ] * w[k][BZ]);
   }
@@ -199,11 +201,11 @@ __device__ __forceinline__ void hllc_flux(const T* a, const T* b, const Phys<T>&
     for (int v = 0; v < NV; ++v) f[v] = F[1][v];
   } else {
     const T ra = w[0][RHO], rb = w[1][RHO];
-    const T sm = (rb * u[1] * (sr - u[1]) - ra * u[0] * (sl - u[0]) - pt[1] + pt[0]) /
-                 (rb * (sr - u[1]) - ra * (sl - u[0]));
+    const T sm = qdiv<T>(rb * u[1] * (sr - u[1]) - ra * u[0] * (sl - u[0]) - pt[1] + pt[0],
+                         rb * (sr - u[1]) - ra * (sl - u[0]));
     constexpr int T1 = D == 0 ? 1 : 0, T2 = D == 2 ? 1 : 2;   // tangential dimensions
-    const T bt1 = (sr * w[1][BX + T1] - sl * w[0][BX + T1] - (F[1][BX + T1] - F[0][BX + T1])) / (sr - sl);
-    const T bt2 = (sr * w[1][BX + T2] - sl * w[0][BX + T2] - (F[1][BX + T2] - F[0][BX + T2])) / (sr - sl);
+    const T bt1 = qdiv<T>(sr * w[1][BX + T1] - sl * w[0][BX + T1] - (F[1][BX + T1] - F[0][BX + T1]), sr - sl);
+    const T bt2 = qdiv<T>(sr * w[1][BX + T2] - sl * w[0][BX + T2] - (F[1][BX + T2] - F[0][BX + T2]), sr - sl);
     const int k = sm >= T(0) ? 0 : 1;
     const T sk = k ? sr : sl;
     T wk[NV], Fk[NV];
@@ -214,21 +216,21 @@ __device__ __forceinline__ void hllc_flux(const T* a, const T* b, const Phys<T>&
     }
     const T uk = k ? u[1] : u[0], ptk = k ? pt[1] : pt[0];
     const T dk = sk - uk, ds = sk - sm;
-    const T rs = wk[RHO] * dk / ds;
+    const T rs = qdiv<T>(wk[RHO] * dk, ds);
     const T pts = ptk + wk[RHO] * dk * (sm - uk);
-    const T vbk = (wk[MX] / wk[RHO]) * wk[BX] + (wk[MX + 1] / wk[RHO]) * wk[BY] + (wk[MX + 2] / wk[RHO]) * wk[BZ];
+    const T vbk = qdiv<T>(wk[MX], wk[RHO]) * wk[BX] + qdiv<T>(wk[MY], wk[RHO]) * wk[BY] + qdiv<T>(wk[MZ], wk[RHO]) * wk[BZ];
     T us[NV];
     us[RHO] = rs;
     us[MX + D] = rs * sm;
-    us[MX + T1] = rs * (wk[MX + T1] / wk[RHO]) - bm * (bt1 - wk[BX + T1]) / ds;
-    us[MX + T2] = rs * (wk[MX + T2] / wk[RHO]) - bm * (bt2 - wk[BX + T2]) / ds;
+    us[MX + T1] = rs * qdiv<T>(wk[MX + T1], wk[RHO]) - qdiv<T>(bm * (bt1 - wk[BX + T1]), ds);
+    us[MX + T2] = rs * qdiv<T>(wk[MX + T2], wk[RHO]) - qdiv<T>(bm * (bt2 - wk[BX + T2]), ds);
     T vbs = sm * bm;
-    vbs += (us[MX + T1] / rs) * bt1;
-    vbs += (us[MX + T2] / rs) * bt2;
+    vbs += qdiv<T>(us[MX + T1], rs) * bt1;
+    vbs += qdiv<T>(us[MX + T2], rs) * bt2;
     us[BX + D] = bm;
     us[BX + T1] = bt1;
     us[BX + T2] = bt2;
-    us[EN] = (wk[EN] * dk - ptk * uk + pts * sm + bm * (vbk - vbs)) / ds;
+    us[EN] = qdiv<T>(wk[EN] * dk - ptk * uk + pts * sm + bm * (vbk - vbs), ds);
     us[PSI] = wk[PSI];
 #pragma unroll
     for (int v = 0; v < NV; ++v) f[v] = Fk[v] + sk * (us[v] - wk[v]);
@@ -259,7 +261,7 @@ __device__ __forceinline__ void hllc_flux(const T* a, const T* b, const Phys<T>&
 template <typename T, int D>
 __device__ __forceinline__ void hlld_flux(const T* a, const T* b, const Phys<T>& P, T* f) {
   const T ch = P.ch;
-  const T bm = ch > T(0) ? T(0.5) * (a[BX + D] + b[BX + D]) - (b[PSI] - a[PSI]) / (T(2) * ch)
+  const T bm = ch > T(0) ? T(0.5) * (a[BX + D] + b[BX + D]) - qdiv<T>(b[PSI] - a[PSI], T(2) * ch)
                          : T(0.5) * (a[BX + D] + b[BX + D]);
   T w[2][NV], F[2][NV], u[2], cf[2], pt[2];
 #pragma unroll
@@ -272,7 +274,7 @@ __device__ __forceinline__ void hlld_flux(const T* a, const T* b, const Phys<T>&
     w[k][EN] = q[EN] + T(0.5) * (bm * bm - q[BX + D] * q[BX + D]);
     const T pw = pressure<T>(w[k], P);
     flux_p<T, D>(w[k], pw, P, F[k]);
-    u[k] = w[k][MX + D] / w[k][RHO];
+    u[k] = qdiv<T>(w[k][MX + D], w[k][RHO]);
     cf[k] = fast_speed<T, D>(w[k], pw, P);
     pt[k] = p + T(0.5) * (w[k][BX] * w[k][BX] + w[k][BY] * w[k][BY] + w[k][BZ] * w[k][BZ]);
   }
@@ -289,15 +291,15 @@ __device__ __forceinline__ void hlld_flux(const T* a, const T* b, const Phys<T>&
     const T dl = sl - u[0], dr = sr - u[1];
     const T ra = w[0][RHO], rb = w[1][RHO];
     const T den = dr * rb - dl * ra;
-    const T sm = (dr * rb * u[1] - dl * ra * u[0] - pt[1] + pt[0]) / den;
-    const T pts = (dr * rb * pt[0] - dl * ra * pt[1] + ra * rb * dr * dl * (u[1] - u[0])) / den;
+    const T sm = qdiv<T>(dr * rb * u[1] - dl * ra * u[0] - pt[1] + pt[0], den);
+    const T pts = qdiv<T>(dr * rb * pt[0] - dl * ra * pt[1] + ra * rb * dr * dl * (u[1] - u[0]), den);
     // outer-state velocity and field (absolute components), density, v*.B*, both sides
     T vs[2][3], bs[2][3], rs[2], vbs[2];
     const T tiny = sizeof(T) == 4 ? T(1e-6) : T(1e-12);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const T rho = w[k][RHO], dk = (k ? sr : sl) - u[k], ds = (k ? sr : sl) - sm;
-      rs[k] = rho * dk / ds;
+      rs[k] = qdiv<T>(rho * dk, ds);
       const T Dk = rho * dk * ds - bm * bm;
       const bool flat = fabs(Dk) <= tiny * (fabs(rho * dk * ds) + bm * bm);
       vs[k][D] = sm;
@@ -305,9 +307,9 @@ __device__ __forceinline__ void hlld_flux(const T* a, const T* b, const Phys<T>&
 #pragma unroll
       for (int t = 0; t < 2; ++t) {
         const int j = t ? T2 : T1;
-        const T vt = w[k][MX + j] / rho, bt = w[k][BX + j];
-        vs[k][j] = flat ? vt : vt - bm * bt * (sm - u[k]) / Dk;
-        bs[k][j] = flat ? bt : bt * (rho * dk * dk - bm * bm) / Dk;
+        const T vt = qdiv<T>(w[k][MX + j], rho), bt = w[k][BX + j];
+        vs[k][j] = flat ? vt : vt - qdiv<T>(bm * bt * (sm - u[k]), Dk);
+        bs[k][j] = flat ? bt : qdiv<T>(bt * (rho * dk * dk - bm * bm), Dk);
       }
       vbs[k] = vs[k][0] * bs[k][0] + vs[k][1] * bs[k][1] + vs[k][2] * bs[k][2];
     }
@@ -324,7 +326,7 @@ __device__ __forceinline__ void hlld_flux(const T* a, const T* b, const Phys<T>&
     const T rsk = k ? rs[1] : rs[0], vbsk = k ? vbs[1] : vbs[0];
     T vb = T(0);
 #pragma unroll
-    for (int j = 0; j < 3; ++j) vb += (wk[MX + j] / wk[RHO]) * wk[BX + j];
+    for (int j = 0; j < 3; ++j) vb += qdiv<T>(wk[MX + j], wk[RHO]) * wk[BX + j];
     T us[NV];
     us[RHO] = rsk;
 #pragma unroll
@@ -332,11 +334,11 @@ __device__ __forceinline__ void hlld_flux(const T* a, const T* b, const Phys<T>&
       us[MX + j] = rsk * (k ? vs[1][j] : vs[0][j]);
       us[BX + j] = k ? bs[1][j] : bs[0][j];
     }
-    us[EN] = (dk * wk[EN] - ptk * uk + pts * sm + bm * (vb - vbsk)) / ds;
+    us[EN] = qdiv<T>(dk * wk[EN] - ptk * uk + pts * sm + bm * (vb - vbsk), ds);
     us[PSI] = wk[PSI];
     const T sgn = bm > T(0) ? T(1) : (bm < T(0) ? T(-1) : T(0));
     const T rl = sqrt(rs[0]), rr = sqrt(rs[1]);
-    const T ssk = k ? sm + fabs(bm) / rr : sm - fabs(bm) / rl;
+    const T ssk = k ? sm + qdiv<T>(fabs(bm), rr) : sm - qdiv<T>(fabs(bm), rl);
     // left of the contact the inner region lies right of S*_L, right of it left of S*_R
     const bool inner = k ? ssk >= T(0) : ssk < T(0);
     if (inner) {
@@ -346,8 +348,8 @@ __device__ __forceinline__ void hlld_flux(const T* a, const T* b, const Phys<T>&
 #pragma unroll
       for (int t = 0; t < 2; ++t) {
         const int j = t ? T2 : T1;
-        vss[j] = (rl * vs[0][j] + rr * vs[1][j] + sgn * (bs[1][j] - bs[0][j])) / (rl + rr);
-        bss[j] = (rl * bs[1][j] + rr * bs[0][j] + sgn * rl * rr * (vs[1][j] - vs[0][j])) / (rl + rr);
+        vss[j] = qdiv<T>(rl * vs[0][j] + rr * vs[1][j] + sgn * (bs[1][j] - bs[0][j]), rl + rr);
+        bss[j] = qdiv<T>(rl * bs[1][j] + rr * bs[0][j] + sgn * rl * rr * (vs[1][j] - vs[0][j]), rl + rr);
       }
       const T vbss = vss[0] * bss[0] + vss[1] * bss[1] + vss[2] * bss[2];
       T uss[NV];
