@@ -435,10 +435,12 @@ class Pool:
         """The new leaf list (n, 5) decided from per-leaf flags (map_plan_regrid)."""
         f = np.ascontiguousarray(flags, dtype=np.int8)
         cap = int(self.nleaves * (8 if self.mesh.ndim == 3 else 4))
-        arr = (map_block_desc * cap)()
+        out = np.empty((cap, 5), dtype=np.int32)         # map_block_desc is five packed int32
         n = C.c_int(0)
-        self._ck(load().map_plan_regrid(self.h, _ptr(f), int(max_level), arr, cap, C.byref(n)), "map_plan_regrid")
-        return _leaves_to_array(arr, n.value)
+        self._ck(load().map_plan_regrid(self.h, _ptr(f), int(max_level),
+                                        out.ctypes.data_as(C.POINTER(map_block_desc)), cap, C.byref(n)),
+                 "map_plan_regrid")
+        return out[:n.value].copy()
 
     def get_leaves(self) -> np.ndarray:
         cap = self.nleaves

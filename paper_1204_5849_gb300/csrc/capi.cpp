@@ -11,20 +11,53 @@
 
 using namespace mapgb;
 
+// A device array that is kept from tree to tree and grown when a larger one needs it.
+template <typename X>
+struct DevArray {
+  X* p = nullptr;
+  size_t cap = 0;
+  operator X*() const { return p; }
+  cudaError_t reserve(size_t n) {
+    if (n <= cap) return cudaSuccess;
+    release();
+    const size_t want = n + n / 4;
+    cudaError_t e = cudaMalloc((void**)&p, want * sizeof(X));
+    if (e != cudaSuccess) {             // no room to spare: the size itself
+      cudaGetLastError();
+      e = cudaMalloc((void**)&p, n * sizeof(X));
+      if (e == cudaSuccess) cap = n;
+      else p = nullptr;
+      return e;
+    }
+    cap = want;
+    return e;
+  }
+  cudaError_t upload(const std::vector<X>& src, cudaStream_t s) {
+    cudaError_t e = reserve(src.size() ? src.size() : 1);
+    if (e != cudaSuccess || src.empty()) return e;
+    return cudaMemcpyAsync(p, src.data(), src.size() * sizeof(X), cudaMemcpyHostToDevice, s);
+  }
+  void release() {
+    cudaFree(p);
+    p = nullptr;
+    cap = 0;
+  }
+};
+
 struct DevTree {
-  BlockGeo* geo = nullptr;
-  GhostRegion* regions = nullptr;
-  int* children = nullptr;
-  int* leaf_ids = nullptr;     // caller leaf order -> pool id
-  int* all_leaves = nullptr;   // pool ids 0..n-1 (Morton order)
-  int* level_leaves = nullptr; // concatenated by level
-  int* level_parents = nullptr;
-  int* level_residual = nullptr;  // per level: leaves with ghost regions the pushes leave over
-  PushEntry* pushes = nullptr;
-  RefluxLeaf* refl = nullptr;
-  RefluxTask* rtasks = nullptr;
+  DevArray<BlockGeo> geo;
+  DevArray<GhostRegion> regions;
+  DevArray<int> children;
+  DevArray<int> leaf_ids;      // caller leaf order -> pool id
+  DevArray<int> all_leaves;    // pool ids 0..n-1 (Morton order)
+  DevArray<int> level_leaves;  // concatenated by level
+  DevArray<int> level_parents;
+  DevArray<int> level_residual;   // per level: leaves with ghost regions the pushes leave over
+  DevArray<PushEntry> pushes;
+  DevArray<RefluxLeaf> refl;
+  DevArray<RefluxTask> rtasks;
   int nrtasks = 0;
-  void* freg = nullptr;        // face registers, tree.nslots slots
+  DevArray<char> freg;         // face registers, tree.nslots slots
   std::vector<int> leaf_off, parent_off, residual_off;  // offsets per level (host)
   // partitioned pools (map_set_active): the leaves this pool steps, reduces and sums
   int* act_all = nullptr;      // pool ids, Morton order
@@ -147,25 +180,35 @@ static bool is64(const map_pool* p) { return p->precision == MAP_FP64; }
   (is64(pool) ? launch_##name##_f64(kcfg(pool), L, pool->stream, &pool->launches) \
               : launch_##name##_f32(kcfg(pool), L, pool->stream, &pool->launches))
 
-static void free_tree(map_pool* pool) {
-  cudaFree(pool->dt.geo);
-  cudaFree(pool->dt.regions);
-  cudaFree(pool->dt.children);
-  cudaFree(pool->dt.leaf_ids);
-  cudaFree(pool->dt.all_leaves);
-  cudaFree(pool->dt.level_leaves);
-  cudaFree(pool->dt.level_parents);
-  cudaFree(pool->dt.level_residual);
-  cudaFree(pool->dt.pushes);
-  cudaFree(pool->dt.refl);
-  cudaFree(pool->dt.rtasks);
-  cudaFree(pool->dt.freg);
-  cudaFree(pool->dt.act_all);
-  cudaFree(pool->dt.act_level);
-  cudaFree(pool->dt.xfer_ids);
-  cudaFree(pool->dt.chunk_ids);
-  pool->dt = DevTree();
+// What belongs to one tree only: the active leaves, the transfer ids and the chunk list.  The
+// tables stay for the next tree (sixteen frees and allocations took 0.25 ms of a regrid).
+static void forget_tree(map_pool* pool) {
+  DevTree& D = pool->dt;
+  cudaFree(D.act_all);
+  cudaFree(D.act_level);
+  cudaFree(D.xfer_ids);
+  cudaFree(D.chunk_ids);
+  D.act_all = D.act_level = D.xfer_ids = D.chunk_ids = nullptr;
+  D.n_act = D.nrtasks = D.chunk_grid = 0;
+  D.chunk_partial = false;
   pool->partial = false;
+}
+
+static void free_tree(map_pool* pool) {
+  forget_tree(pool);
+  DevTree& D = pool->dt;
+  D.geo.release();
+  D.regions.release();
+  D.children.release();
+  D.leaf_ids.release();
+  D.all_leaves.release();
+  D.level_leaves.release();
+  D.level_parents.release();
+  D.level_residual.release();
+  D.pushes.release();
+  D.refl.release();
+  D.rtasks.release();
+  D.freg.release();
 }
 
 static void drop_graphs(map_pool* pool) {
@@ -307,21 +350,22 @@ int map_set_stream(map_pool* pool, void* stream) {
 }
 
 static int install_tree(map_pool* pool, HostTree& t) {
-  free_tree(pool);
+  forget_tree(pool);
   drop_graphs(pool);
   pool->cond_copies = -1;
   DevTree& D = pool->dt;
-  CK(upload(&D.geo, t.geo, pool->stream));
-  CK(upload(&D.regions, t.regions, pool->stream));
-  CK(upload(&D.children, t.children, pool->stream));
-  CK(upload(&D.leaf_ids, t.leaf_to_block, pool->stream));
-  CK(upload(&D.all_leaves, t.all_leaves, pool->stream));
-  CK(upload(&D.pushes, t.pushes, pool->stream));
-  CK(upload(&D.refl, t.refl, pool->stream));
+  // (stream-ordered behind the kernels that read the tables before)
+  CK(D.geo.upload(t.geo, pool->stream));
+  CK(D.regions.upload(t.regions, pool->stream));
+  CK(D.children.upload(t.children, pool->stream));
+  CK(D.leaf_ids.upload(t.leaf_to_block, pool->stream));
+  CK(D.all_leaves.upload(t.all_leaves, pool->stream));
+  CK(D.pushes.upload(t.pushes, pool->stream));
+  CK(D.refl.upload(t.refl, pool->stream));
   if (!t.reflux_tasks.empty()) {
-    CK(upload(&D.rtasks, t.reflux_tasks, pool->stream));
+    CK(D.rtasks.upload(t.reflux_tasks, pool->stream));
     D.nrtasks = (int)t.reflux_tasks.size();
-    CK(cudaMalloc(&D.freg, (size_t)t.nslots * 2 * pool->ndim * kNV * pool->nb * pool->nb * pool->elem));
+    CK(D.freg.reserve((size_t)t.nslots * 2 * pool->ndim * kNV * pool->nb * pool->nb * pool->elem));
   }
   std::vector<int> ll, pl, rl;
   D.leaf_off.assign(t.maxlev + 2, 0);
@@ -338,9 +382,9 @@ static int install_tree(map_pool* pool, HostTree& t) {
   D.leaf_off[t.maxlev + 1] = (int)ll.size();
   D.parent_off[t.maxlev + 1] = (int)pl.size();
   D.residual_off[t.maxlev + 1] = (int)rl.size();
-  CK(upload(&D.level_leaves, ll, pool->stream));
-  CK(upload(&D.level_parents, pl, pool->stream));
-  CK(upload(&D.level_residual, rl, pool->stream));
+  CK(D.level_leaves.upload(ll, pool->stream));
+  CK(D.level_parents.upload(pl, pool->stream));
+  CK(D.level_residual.upload(rl, pool->stream));
   // per-problem minimum spacing (dt uses the finest leaf, Sec. 4.5 / Sec. 3.7)
   std::vector<ProbDyn> dyn(pool->nprob);
   CK(cudaMemcpyAsync(dyn.data(), pool->dyn, sizeof(ProbDyn) * pool->nprob, cudaMemcpyDeviceToHost, pool->stream));
@@ -624,7 +668,7 @@ static int alpha_device(map_pool* pool, const map_params* p) {
   CK(launch_zero_alpha(pool->dyn, pool->nprob, pool->stream, &pool->launches));
   CflLaunch C;
   C.u = pool->buf[pool->cur];
-  C.blocks = pool->partial ? pool->dt.act_all : pool->dt.all_leaves;
+  C.blocks = pool->partial ? pool->dt.act_all : pool->dt.all_leaves.p;
   C.nblocks = pool->partial ? pool->dt.n_act : pool->tree.nleaves;
   C.geo = pool->dt.geo;
   C.dyn = pool->dyn;
@@ -745,7 +789,7 @@ static int step_block_list(map_pool* pool, int G, const int** list) {
   DevTree& D = pool->dt;
   const HostTree& t = pool->tree;
   const int n = pool->partial ? D.n_act : t.nleaves;
-  *list = pool->partial ? D.act_all : D.all_leaves;
+  *list = pool->partial ? D.act_all : D.all_leaves.p;
   if (G <= 0 || G >= n) return MAP_OK;
   if (D.chunk_ids && D.chunk_grid == G && D.chunk_partial == pool->partial) {
     *list = D.chunk_ids;
@@ -793,8 +837,8 @@ static int step_launches(map_pool* pool, const map_params* p, bool fused) {
   S.dyn_next = fused ? pool->dyn : nullptr;
   S.pushes = pool->dt.pushes;
   const bool reflux = p->reflux != 0 && pool->dt.nrtasks > 0;
-  S.freg = reflux ? pool->dt.freg : nullptr;
-  S.refl = reflux ? pool->dt.refl : nullptr;
+  S.freg = reflux ? (void*)pool->dt.freg.p : nullptr;
+  S.refl = reflux ? pool->dt.refl.p : nullptr;
   const int in = pool->cur, out = 1 - pool->cur;
   // the plain FP64 form launches once per level; the FP32 form once over all leaves
   auto run = [&](const void* uin, void* uout, const void* ubase, int stage, bool with_fused) -> int {
@@ -808,7 +852,7 @@ static int step_launches(map_pool* pool, const map_params* p, bool fused) {
     if (is64(pool)) {
       for (int L = 0; L <= t.maxlev; ++L) {
         const std::vector<int>& off = pool->partial ? D.act_off : D.leaf_off;
-        S.blocks = (pool->partial ? D.act_level : D.level_leaves) + off[L];
+        S.blocks = (pool->partial ? D.act_level : D.level_leaves.p) + off[L];
         S.nblocks = off[L + 1] - off[L];
         if (S.nblocks == 0) continue;
         S.grid = pool->tune_grid;
@@ -1049,8 +1093,8 @@ static int conduction_substep(map_pool* pool, const map_params* p, int it, bool 
     C.hsub = pool->hsub;
     C.nsub = pool->nsub;
     C.it = it;
-    C.freg = rf ? pool->dt.freg : nullptr;
-    C.refl = rf ? pool->dt.refl : nullptr;
+    C.freg = rf ? (void*)pool->dt.freg.p : nullptr;
+    C.refl = rf ? pool->dt.refl.p : nullptr;
     CK(DISPATCH(pool, conduction, C));
     if (rf) {
       RefluxLaunch R;
@@ -1229,7 +1273,7 @@ int map_plan_regrid(map_pool* pool, const int8_t* flags, int max_level, map_bloc
   if (!pool || !flags || !n_out) return fail(pool, MAP_EINVAL, "null argument");
   if (!pool->have_tree) return fail(pool, MAP_ESTATE, "no tree");
   std::vector<map_block_desc> plan;
-  std::string why = plan_regrid(pool->tree, pool->probs, flags, max_level, plan);
+  std::string why = plan_regrid(pool->tree, flags, max_level, plan);
   if (!why.empty()) return fail(pool, MAP_EINVAL, why);
   *n_out = (int)plan.size();
   if ((int)plan.size() > cap || !out) return fail(pool, MAP_ENOMEM, "output array too small for the new leaf list");
@@ -1261,7 +1305,7 @@ int map_adapt(map_pool* pool, const map_params* p, const map_refine_params* r, i
   rc = map_flag_refine(pool, p, r, flags.data(), nullptr);
   if (rc) return rc;
   std::vector<map_block_desc> plan;
-  std::string why = plan_regrid(pool->tree, pool->probs, flags.data(), r->max_level, plan);
+  std::string why = plan_regrid(pool->tree, flags.data(), r->max_level, plan);
   if (!why.empty()) return fail(pool, MAP_EINVAL, why);
   bool same = (int)plan.size() == pool->tree.nleaves;
   for (int l = 0; same && l < pool->tree.nleaves; ++l) {
@@ -1281,7 +1325,7 @@ int map_conservation(map_pool* pool, double* sums_out) {
   CK(cudaMemsetAsync(pool->sums, 0, sizeof(double) * kNV * pool->nprob, pool->stream));
   SumLaunch L;
   L.u = pool->buf[pool->cur];
-  L.blocks = pool->partial ? pool->dt.act_all : pool->dt.all_leaves;
+  L.blocks = pool->partial ? pool->dt.act_all : pool->dt.all_leaves.p;
   L.nblocks = pool->partial ? pool->dt.n_act : pool->tree.nleaves;
   L.geo = pool->dt.geo;
   L.sums = pool->sums;
@@ -1511,7 +1555,7 @@ int map_plan_leaves(int ndim, int nb, const map_problem_desc* problems, int n_pr
   std::vector<map_problem_desc> probs;
   std::string why = host_tree(ndim, nb, problems, n_problems, leaves, n, t, probs);
   std::vector<map_block_desc> plan;
-  if (why.empty()) why = plan_regrid(t, probs, flags, max_level, plan);
+  if (why.empty()) why = plan_regrid(t, flags, max_level, plan);
   if (!why.empty()) {
     put_msg(msg, msg_cap, why);
     return MAP_EINVAL;

@@ -93,8 +93,12 @@ struct HostTree {
   std::vector<BlockGeo> geo;                // per pool block
   std::vector<int> blk_problem, blk_level, blk_ijk;  // ijk: 3 per block
   std::vector<int> children;                // 8 per block (-1 if leaf)
-  std::vector<GhostRegion> regions;         // 27 per block (valid for leaves)
-  std::vector<PushEntry> pushes;            // 27 per block (valid for leaves)
+  std::vector<int> parent;                  // per block (-1 at level 0)
+  // per leaf and direction (dx+1) + 3(dy+1) + 9(dz+1), periodic wrap: the same-level block there
+  // (a leaf or a parent), -2 - id of the coarser leaf covering it, or -1 outside the domain
+  std::vector<int> nbr;
+  std::vector<GhostRegion> regions;         // 27 per leaf (2D: rz = 1 only)
+  std::vector<PushEntry> pushes;            // 27 per leaf
   std::vector<char> level_has_residual;     // per level: a ghost region the fill must do
   std::vector<RefluxLeaf> refl;             // per block
   std::vector<RefluxTask> reflux_tasks;     // per coarse leaf at a coarse/fine face
@@ -107,8 +111,8 @@ struct HostTree {
   std::vector<int> leaves_per_problem;
   // lookup (problem, level, i, j, k) -> pool id
   int find(int p, int L, int i, int j, int k) const;
-  std::vector<std::pair<unsigned long long, int>> keys;  // sorted packed keys -> id
-  // open-addressing hash index over the same keys (linear probing, power-of-two table)
+  std::vector<std::pair<unsigned long long, int>> keys;  // packed keys -> id
+  // open-addressing hash index over them (linear probing, power-of-two table)
   std::vector<unsigned long long> hkeys;
   std::vector<int> hvals;
   unsigned long long hmask = 0;
@@ -127,7 +131,7 @@ std::string build_tree(int ndim, int nb, const std::vector<map_problem_desc>& pr
 
 // Regrid decision from per-leaf flags (+1 refine, 0 keep, -1 may coarsen); the new leaf
 // list in the documented order.  Empty string on success.
-std::string plan_regrid(const HostTree& t, const std::vector<map_problem_desc>& probs, const int8_t* flags,
+std::string plan_regrid(const HostTree& t, const int8_t* flags,
                         int max_level, std::vector<map_block_desc>& out);
 
 // Partition of the leaves over nranks (Morton ranges of equal count, Sec. 4.2) and, per

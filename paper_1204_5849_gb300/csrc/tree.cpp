@@ -24,22 +24,27 @@ unsigned long long pack_key(int p, int L, int i, int j, int k) {
          ((unsigned long long)k << 30) | ((unsigned long long)j << 15) | (unsigned long long)i;
 }
 
+// bits of x moved apart by doubling the gaps (one mask per step): bit q -> bit 2q or 3q
+unsigned long long spread2(unsigned long long x) {
+  x &= 0xffffffffull;
+  x = (x | (x << 16)) & 0x0000ffff0000ffffull;
+  x = (x | (x << 8)) & 0x00ff00ff00ff00ffull;
+  x = (x | (x << 4)) & 0x0f0f0f0f0f0f0f0full;
+  x = (x | (x << 2)) & 0x3333333333333333ull;
+  return (x | (x << 1)) & 0x5555555555555555ull;
+}
+
 unsigned long long spread3(unsigned long long x) {
-  // bit q of x -> bit 3q
-  unsigned long long r = 0;
-  for (int q = 0; q < 21; ++q) r |= ((x >> q) & 1ull) << (3 * q);
-  return r;
+  x &= 0x1fffffull;
+  x = (x | (x << 32)) & 0x001f00000000ffffull;
+  x = (x | (x << 16)) & 0x001f0000ff0000ffull;
+  x = (x | (x << 8)) & 0x100f00f00f00f00full;
+  x = (x | (x << 4)) & 0x10c30c30c30c30c3ull;
+  return (x | (x << 2)) & 0x1249249249249249ull;
 }
 
 unsigned long long morton(int ndim, int i, int j, int k) {
-  if (ndim == 2) {
-    unsigned long long r = 0;
-    for (int q = 0; q < 31; ++q) {
-      r |= ((unsigned long long)((i >> q) & 1) << (2 * q));
-      r |= ((unsigned long long)((j >> q) & 1) << (2 * q + 1));
-    }
-    return r;
-  }
+  if (ndim == 2) return spread2((unsigned)i) | (spread2((unsigned)j) << 1);
   return spread3(i) | (spread3(j) << 1) | (spread3(k) << 2);
 }
 
@@ -117,12 +122,11 @@ unsigned long long mix64(unsigned long long x) {
 void HostTree::reset() {
   ndim = nb = nblocks = nleaves = maxlev = nslots = 0;
   hmask = 0;
-  for (auto* v : {&leaf_to_block, &blk_problem, &blk_level, &blk_ijk, &children, &all_leaves, &leaves_per_problem,
-                  &hvals})
+  for (auto* v : {&leaf_to_block, &blk_problem, &blk_level, &blk_ijk, &children, &parent, &all_leaves,
+                  &leaves_per_problem, &hvals})
     v->clear();
   geo.clear();
-  regions.clear();
-  pushes.clear();
+  pushes.clear();      // (regions and nbr are written for every leaf: their storage is kept)
   level_has_residual.clear();
   refl.clear();
   reflux_tasks.clear();
@@ -150,17 +154,44 @@ void HostTree::build_index() {
 
 int HostTree::find(int p, int L, int i, int j, int k) const {
   if (i < 0 || j < 0 || k < 0 || i >= (1 << 15) || j >= (1 << 15) || k >= (1 << 15)) return -1;
+  if (hkeys.empty()) return -1;
   const unsigned long long key = pack_key(p, L, i, j, k);
-  if (hkeys.empty()) {
-    auto it = std::lower_bound(keys.begin(), keys.end(), std::make_pair(key, -1));
-    return (it != keys.end() && it->first == key) ? it->second : -1;
-  }
   unsigned long long h = mix64(key) & hmask;
   while (hkeys[h] != kEmpty) {
     if (hkeys[h] == key) return hvals[h];
     h = (h + 1) & hmask;
   }
   return -1;
+}
+
+// Why the first n nodes (leaves) overlap: a leaf listed twice, or one that contains another (the
+// first in key order of the leaves, else of the ancestors).
+static std::string overlap_message(const std::vector<Node>& nodes, int n,
+                                   std::vector<std::pair<unsigned long long, int>> keys) {
+  std::sort(keys.begin(), keys.end());
+  for (size_t q = 1; q < keys.size(); ++q)
+    if (keys[q].first == keys[q - 1].first) {
+      const Node& lf = nodes[keys[q].second];
+      return fmt("duplicate leaf", lf.p, lf.L, lf.ijk);
+    }
+  std::vector<unsigned long long> anc;
+  for (int l = 0; l < n; ++l) {
+    Node c = nodes[l];
+    while (c.L > 0) {
+      c.L -= 1;
+      for (int d = 0; d < 3; ++d) c.ijk[d] >>= 1;
+      anc.push_back(pack_key(c.p, c.L, c.ijk[0], c.ijk[1], c.ijk[2]));
+    }
+  }
+  std::sort(anc.begin(), anc.end());
+  for (const unsigned long long k : anc) {
+    auto it = std::lower_bound(keys.begin(), keys.end(), std::make_pair(k, -1));
+    if (it != keys.end() && it->first == k) {
+      const Node& lf = nodes[it->second];
+      return fmt("leaf contains another leaf", lf.p, lf.L, lf.ijk);
+    }
+  }
+  return "overlapping leaves";
 }
 
 std::string build_tree(int ndim, int nb, const std::vector<map_problem_desc>& probs,
@@ -201,57 +232,80 @@ std::string build_tree(int ndim, int nb, const std::vector<map_problem_desc>& pr
     keys.push_back({pack_key(nd.p, nd.L, nd.ijk[0], nd.ijk[1], nd.ijk[2]), (int)nodes.size()});
     nodes.push_back(nd);
   }
-  std::sort(keys.begin(), keys.end());
-  for (size_t q = 1; q < keys.size(); ++q)
-    if (keys[q].first == keys[q - 1].first) return fmt("duplicate leaf", nodes[keys[q].second].p,
-                                                       nodes[keys[q].second].L, nodes[keys[q].second].ijk);
-  // ancestors
-  std::vector<std::pair<unsigned long long, int>> anc;
-  for (int l = 0; l < n; ++l) {
-    Node c = nodes[l];
-    while (c.L > 0) {
-      c.L -= 1;
-      for (int d = 0; d < 3; ++d) c.ijk[d] >>= 1;
-      anc.push_back({pack_key(c.p, c.L, c.ijk[0], c.ijk[1], c.ijk[2]), l});
+  // duplicates and ancestors through a hash of the nodes' keys: a leaf's ancestors are added up
+  // to the first that is there already (its own ancestors are, too)
+  {
+    size_t cap = 16;
+    while (cap < 4 * keys.size()) cap <<= 1;
+    std::vector<unsigned long long> hk(cap, kEmpty);
+    std::vector<int> hv(cap, -1);
+    size_t used = 0;
+    // the slot of a key, or the free slot where it goes
+    auto slot = [&](unsigned long long key) {
+      size_t h = mix64(key) & (cap - 1);
+      while (hk[h] != kEmpty && hk[h] != key) h = (h + 1) & (cap - 1);
+      return h;
+    };
+    auto put = [&](size_t h, unsigned long long key, int v) {
+      hk[h] = key;
+      hv[h] = v;
+      if (2 * ++used <= cap) return;
+      std::vector<unsigned long long> ok(cap * 2, kEmpty);
+      std::vector<int> ov(cap * 2, -1);
+      ok.swap(hk);
+      ov.swap(hv);
+      cap *= 2;
+      for (size_t q = 0; q < ok.size(); ++q)
+        if (ok[q] != kEmpty) {
+          const size_t s = slot(ok[q]);
+          hk[s] = ok[q];
+          hv[s] = ov[q];
+        }
+    };
+    bool bad = false;
+    for (int l = 0; l < n && !bad; ++l) {
+      const size_t h = slot(keys[l].first);
+      if (hk[h] != kEmpty) bad = true;
+      else put(h, keys[l].first, l);
     }
-  }
-  std::sort(anc.begin(), anc.end());
-  for (size_t q = 0; q < anc.size(); ++q) {
-    if (q > 0 && anc[q].first == anc[q - 1].first) continue;
-    auto it = std::lower_bound(keys.begin(), keys.end(), std::make_pair(anc[q].first, -1));
-    if (it != keys.end() && it->first == anc[q].first) {
-      const Node& lf = nodes[it->second];
-      return fmt("leaf contains another leaf", lf.p, lf.L, lf.ijk);
+    for (int l = 0; l < n && !bad; ++l) {
+      Node c = nodes[l];
+      c.leaf = false;
+      c.caller = -1;
+      while (c.L > 0) {
+        c.L -= 1;
+        for (int d = 0; d < 3; ++d) c.ijk[d] >>= 1;
+        const unsigned long long key = pack_key(c.p, c.L, c.ijk[0], c.ijk[1], c.ijk[2]);
+        const size_t h = slot(key);
+        if (hk[h] != kEmpty) {
+          bad = hv[h] < n;
+          break;
+        }
+        put(h, key, (int)nodes.size());
+        nodes.push_back(c);
+      }
     }
-    Node c;
-    unsigned long long k = anc[q].first;
-    c.p = (int)(k >> 50);
-    c.L = (int)((k >> 45) & 31);
-    c.ijk[2] = (int)((k >> 30) & 32767);
-    c.ijk[1] = (int)((k >> 15) & 32767);
-    c.ijk[0] = (int)(k & 32767);
-    c.leaf = false;
-    c.caller = -1;
-    nodes.push_back(c);
+    if (bad) return overlap_message(nodes, n, keys);
   }
-  // pool order: leaves by (problem, Morton at the finest level), then parents by level
-  std::vector<int> order(nodes.size());
-  for (size_t q = 0; q < nodes.size(); ++q) order[q] = (int)q;
+  // pool order: leaves by (problem, Morton at the finest level), then parents by problem and
+  // level, finest first
+  struct Place {
+    unsigned long long mk;
+    int p, L, node;
+  };
   const int ML = t.maxlev;
-  std::vector<unsigned long long> mk(nodes.size());      // Morton key at the finest level
+  std::vector<Place> order(nodes.size());
   for (size_t q = 0; q < nodes.size(); ++q) {
     const Node& a = nodes[q];
     const int s = ML - a.L;
-    mk[q] = morton(ndim, a.ijk[0] << s, a.ijk[1] << s, a.ijk[2] << s);
+    order[q] = Place{morton(ndim, a.ijk[0] << s, a.ijk[1] << s, a.ijk[2] << s), a.p, a.L, (int)q};
   }
-  std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-    const Node& a = nodes[x];
-    const Node& b = nodes[y];
-    if (a.leaf != b.leaf) return a.leaf;
+  const auto by_curve = [](const Place& a, const Place& b) { return a.p != b.p ? a.p < b.p : a.mk < b.mk; };
+  if (!std::is_sorted(order.begin(), order.begin() + n, by_curve)) std::sort(order.begin(), order.begin() + n, by_curve);
+  std::sort(order.begin() + n, order.end(), [](const Place& a, const Place& b) {
     if (a.p != b.p) return a.p < b.p;
-    if (!a.leaf && a.L != b.L) return a.L > b.L;
-    if (mk[x] != mk[y]) return mk[x] < mk[y];
-    return a.L < b.L;
+    if (a.L != b.L) return a.L > b.L;
+    return a.mk < b.mk;
   });
   const int NB = (int)nodes.size();
   t.nblocks = NB;
@@ -265,7 +319,7 @@ std::string build_tree(int ndim, int nb, const std::vector<map_problem_desc>& pr
   t.keys.clear();
   t.keys.reserve(NB);
   for (int id = 0; id < NB; ++id) {
-    const Node& a = nodes[order[id]];
+    const Node& a = nodes[order[id].node];
     t.blk_problem[id] = a.p;
     t.blk_level[id] = a.L;
     for (int d = 0; d < 3; ++d) t.blk_ijk[3 * id + d] = a.ijk[d];
@@ -282,9 +336,9 @@ std::string build_tree(int ndim, int nb, const std::vector<map_problem_desc>& pr
     if (a.leaf) t.leaf_to_block[a.caller] = id;
     t.keys.push_back({pack_key(a.p, a.L, a.ijk[0], a.ijk[1], a.ijk[2]), id});
   }
-  std::sort(t.keys.begin(), t.keys.end());
   t.build_index();
   // parent/child links and completeness
+  t.parent.assign(NB, -1);
   for (int id = 0; id < NB; ++id) {
     int L = t.blk_level[id];
     if (L == 0) continue;
@@ -293,6 +347,7 @@ std::string build_tree(int ndim, int nb, const std::vector<map_problem_desc>& pr
     if (par < 0) return "internal error: missing parent";
     int cb = (c[0] & 1) | ((c[1] & 1) << 1) | ((c[2] & 1) << 2);
     t.children[(size_t)par * 8 + cb] = id;
+    t.parent[id] = par;
   }
   for (int id = n; id < NB; ++id)
     for (int cb = 0; cb < (1 << ndim); ++cb)
@@ -308,32 +363,53 @@ std::string build_tree(int ndim, int nb, const std::vector<map_problem_desc>& pr
             return fmt("domain not covered", p, 0, ijk);
           }
   }
-  // 2:1 balance over faces, edges and corners
+  // One pass over the leaves (on host threads): the neighbours, with 2:1 balance over faces,
+  // edges and corners; from them the ghost regions; and the pushes.  A push -- a same-level leaf
+  // copy with an affine map in every dimension, written by the source block's step kernel into
+  // the destination's ghost region -- goes into a slot of its source: for a fixed region the
+  // same-level neighbour is a translation (with periodic wrap), a bijection, so each (source,
+  // direction) slot belongs to one (destination, region).
+  t.nbr.resize((size_t)n * 27);
+  t.regions.resize((size_t)n * 27);
+  t.pushes.assign((size_t)n * 27, PushEntry{-1, {0, 0, 0}});
+  t.level_has_residual.assign(t.maxlev + 1, 0);
+  t.residual_by_level.assign(t.maxlev + 1, {});
+  std::vector<char> has_residual(n, 0);
+  const int z0 = ndim == 3 ? -1 : 0, z1 = ndim == 3 ? 1 : 0;
   std::string err = for_each_leaf(n, [&](int id) -> std::string {
-    int p = t.blk_problem[id], L = t.blk_level[id];
+    const int p = t.blk_problem[id], L = t.blk_level[id];
     const int* c = &t.blk_ijk[3 * id];
-    for (int oz = (ndim == 3 ? -1 : 0); oz <= (ndim == 3 ? 1 : 0); ++oz)
+    int nblk[3] = {1, 1, 1};
+    for (int d = 0; d < ndim; ++d) nblk[d] = probs[p].nbase[d] << L;
+    int* nbr = &t.nbr[(size_t)id * 27];
+    for (int oz = z0; oz <= z1; ++oz)
       for (int oy = -1; oy <= 1; ++oy)
         for (int ox = -1; ox <= 1; ++ox) {
-          if (!ox && !oy && !oz) continue;
-          int off[3] = {ox, oy, oz}, q[3] = {0, 0, 0};
+          const int off[3] = {ox, oy, oz};
+          int& at = nbr[(ox + 1) + 3 * (oy + 1) + 9 * (oz + 1)];
+          if (!ox && !oy && !oz) {
+            at = id;
+            continue;
+          }
+          int q[3] = {0, 0, 0};
           bool outside = false;
           for (int d = 0; d < ndim; ++d) {
-            int nblk = probs[p].nbase[d] << L;
             q[d] = c[d] + off[d];
-            if (q[d] < 0 || q[d] >= nblk) {
-              if (probs[p].bc[d][q[d] < 0 ? 0 : 1] == MAP_BC_PERIODIC) q[d] = (q[d] + nblk) % nblk;
+            if (q[d] < 0 || q[d] >= nblk[d]) {
+              if (probs[p].bc[d][q[d] < 0 ? 0 : 1] == MAP_BC_PERIODIC) q[d] = (q[d] + nblk[d]) % nblk[d];
               else outside = true;
             }
           }
+          at = -1;
           if (outside) continue;
-          int nbid = t.find(p, L, q[0], q[1], q[2]);
+          const int nbid = t.find(p, L, q[0], q[1], q[2]);
           if (nbid >= 0) {
+            at = nbid;
             if (nbid < n) continue;
             for (int cb = 0; cb < (1 << ndim); ++cb) {
               bool touch = true;
               for (int d = 0; d < ndim; ++d) {
-                int bit = (cb >> d) & 1;
+                const int bit = (cb >> d) & 1;
                 if (off[d] == 1 && bit != 0) touch = false;
                 if (off[d] == -1 && bit != 1) touch = false;
               }
@@ -341,45 +417,42 @@ std::string build_tree(int ndim, int nb, const std::vector<map_problem_desc>& pr
                 return fmt("2:1 balance violated (finer by two levels)", p, L, c);
             }
           } else {
-            int cq = L > 0 ? t.find(p, L - 1, q[0] >> 1, q[1] >> 1, q[2] >> 1) : -1;
+            const int cq = L > 0 ? t.find(p, L - 1, q[0] >> 1, q[1] >> 1, q[2] >> 1) : -1;
             if (cq < 0 || cq >= n) return fmt("2:1 balance violated (coarser by two levels)", p, L, c);
+            at = -2 - cq;
           }
         }
-    return std::string();
-  });
-  if (!err.empty()) return err;
-  // ghost regions of every leaf
-  t.regions.assign((size_t)NB * 27, GhostRegion{});
-  err = for_each_leaf(n, [&](int id) -> std::string {
-    int p = t.blk_problem[id], L = t.blk_level[id];
-    const int* c = &t.blk_ijk[3 * id];
+    bool residual = false;
     for (int rz = 0; rz < 3; ++rz)
       for (int ry = 0; ry < 3; ++ry)
         for (int rx = 0; rx < 3; ++rx) {
           if (ndim == 2 && rz != 1) continue;
-          int r[3] = {rx, ry, rz};
-          int m[3] = {1, 1, 1}, A[3] = {0, 0, 0}, T[3] = {0, 0, 0}, rep[3] = {0, 0, 0};
-          for (int d = 0; d < ndim; ++d) {
-            int N = (probs[p].nbase[d] << L) * nb;
-            int nblk = probs[p].nbase[d] << L;
-            int O = c[d] * nb;
-            int irep = r[d] == 0 ? 0 : (r[d] == 1 ? kNG : kNG + nb);
-            if (r[d] == 1) {
-              m[d] = 1; A[d] = O - kNG; T[d] = c[d];
-            } else {
-              int nbk = c[d] + (r[d] == 0 ? -1 : 1);
-              if (nbk >= 0 && nbk < nblk) {
-                m[d] = 1; A[d] = O - kNG; T[d] = nbk;
-              } else if (probs[p].bc[d][r[d] == 0 ? 0 : 1] == MAP_BC_PERIODIC) {
-                m[d] = 1; A[d] = O - kNG + (r[d] == 0 ? N : -N); T[d] = (nbk + nblk) % nblk;
-              } else {
-                m[d] = 0; A[d] = r[d] == 0 ? 0 : N - 1; T[d] = c[d];
+          const int r[3] = {rx, ry, rz};
+          int m[3] = {1, 1, 1}, A[3] = {0, 0, 0}, T[3] = {0, 0, 0};
+          int dir = 0;                           // direction of the source: 0 where the map clamps
+          for (int d = 0, w = 1; d < 3; ++d, w *= 3) {
+            int o = 0;
+            if (d < ndim) {
+              const int N = nblk[d] * nb, O = c[d] * nb, nbk = c[d] + r[d] - 1;
+              A[d] = O - kNG;
+              T[d] = nbk;
+              o = r[d] - 1;
+              if (nbk < 0 || nbk >= nblk[d]) {
+                if (probs[p].bc[d][r[d] == 0 ? 0 : 1] == MAP_BC_PERIODIC) {
+                  A[d] += r[d] == 0 ? N : -N;
+                  T[d] = (nbk + nblk[d]) % nblk[d];
+                } else {
+                  m[d] = 0;
+                  A[d] = r[d] == 0 ? 0 : N - 1;
+                  T[d] = c[d];
+                  o = 0;
+                }
               }
             }
-            rep[d] = m[d] * irep + A[d];
+            dir += (o + 1) * w;
           }
           GhostRegion g{};
-          int src = t.find(p, L, T[0], T[1], T[2]);
+          const int src = nbr[dir];
           if (src >= 0) {
             g.kind = 0;
             g.src = src;
@@ -389,54 +462,30 @@ std::string build_tree(int ndim, int nb, const std::vector<map_problem_desc>& pr
               g.corg[d] = 0;
             }
           } else {
-            int Tc[3] = {0, 0, 0};
-            for (int d = 0; d < ndim; ++d) Tc[d] = (rep[d] >> 1) / nb;
-            int cs = L > 0 ? t.find(p, L - 1, Tc[0], Tc[1], Tc[2]) : -1;
-            if (cs < 0 || cs >= n) return fmt("no coarse source for a ghost region", p, L, c);
+            if (src == -1) return fmt("no coarse source for a ghost region", p, L, c);
             g.kind = 1;
-            g.src = cs;
+            g.src = -2 - src;
             for (int d = 0; d < 3; ++d) {
               g.m[d] = d < ndim ? m[d] : 1;
               g.a[d] = d < ndim ? A[d] : 0;
-              g.corg[d] = d < ndim ? Tc[d] * nb : 0;
+              g.corg[d] = d < ndim ? (T[d] >> 1) * nb : 0;
             }
           }
-          t.regions[(size_t)id * 27 + rx + 3 * ry + 9 * rz] = g;
-        }
-    return std::string();
-  });
-  if (!err.empty()) return err;
-  // pushes: a same-level leaf copy with an affine map in every dimension is written by the
-  // source block's step kernel into the destination's ghost region
-  // For a fixed region, the same-level neighbour is a translation (with periodic wrap), a
-  // bijection: each (source, direction) slot belongs to one (destination, region), so the
-  // leaves fill their slots independently, on host threads.
-  t.pushes.assign((size_t)NB * 27, PushEntry{-1, {0, 0, 0}});
-  t.level_has_residual.assign(t.maxlev + 1, 0);
-  t.residual_by_level.assign(t.maxlev + 1, {});
-  std::vector<char> has_residual(n, 0);
-  err = for_each_leaf(n, [&](int id) -> std::string {
-    bool residual = false;
-    for (int rz = 0; rz < 3; ++rz)
-      for (int ry = 0; ry < 3; ++ry)
-        for (int rx = 0; rx < 3; ++rx) {
-          if (ndim == 2 && rz != 1) continue;
-          if (rx == 1 && ry == 1 && rz == 1) continue;
-          GhostRegion& g = t.regions[(size_t)id * 27 + rx + 3 * ry + 9 * rz];
-          g.pushed = 0;
-          bool affine = true;
-          for (int d = 0; d < ndim; ++d) affine = affine && g.m[d] == 1;
-          if (g.kind == 0 && affine && g.src < n && t.blk_level[g.src] == t.blk_level[id]) {
-            // seen from the source, this block lies in direction -(r - 1)
-            const int dir = (1 - (rx - 1)) + 3 * (1 - (ry - 1)) + 9 * (ndim == 3 ? 1 - (rz - 1) : 1);
-            PushEntry& pe = t.pushes[(size_t)g.src * 27 + dir];
-            if (pe.dst >= 0) return fmt("internal error: two ghost regions push from one slot", t.blk_problem[id],
-                                        t.blk_level[id], &t.blk_ijk[3 * id]);
-            pe.dst = id;
-            for (int d = 0; d < 3; ++d) pe.off[d] = d < ndim ? -g.a[d] : 0;
-            g.pushed = 1;
+          if (!(rx == 1 && ry == 1 && rz == 1)) {
+            bool affine = true;
+            for (int d = 0; d < ndim; ++d) affine = affine && m[d] == 1;
+            if (g.kind == 0 && affine && g.src < n) {
+              // seen from the source, this block lies in direction -(r - 1)
+              const int back = (1 - (rx - 1)) + 3 * (1 - (ry - 1)) + 9 * (ndim == 3 ? 1 - (rz - 1) : 1);
+              PushEntry& pe = t.pushes[(size_t)g.src * 27 + back];
+              if (pe.dst >= 0) return fmt("internal error: two ghost regions push from one slot", p, L, c);
+              pe.dst = id;
+              for (int d = 0; d < 3; ++d) pe.off[d] = d < ndim ? -g.a[d] : 0;
+              g.pushed = 1;
+            }
+            if (!g.pushed) residual = true;
           }
-          if (!g.pushed) residual = true;
+          t.regions[(size_t)id * 27 + rx + 3 * ry + 9 * rz] = g;
         }
     has_residual[id] = residual ? 1 : 0;
     return std::string();
@@ -464,14 +513,9 @@ std::string build_tree(int ndim, int nb, const std::vector<map_problem_desc>& pr
       bool coarse_side = false;
       for (int d = 0; d < ndim; ++d)
         for (int side = 0; side < 2; ++side) {
-          int q[3] = {c[0], c[1], c[2]};
-          const int nblk = probs[p].nbase[d] << L;
-          q[d] += side ? 1 : -1;
-          if (q[d] < 0 || q[d] >= nblk) {
-            if (probs[p].bc[d][side] != MAP_BC_PERIODIC) continue;
-            q[d] = (q[d] + nblk) % nblk;
-          }
-          const int nbid = t.find(p, L, q[0], q[1], q[2]);
+          const int w[3] = {1, 3, 9};
+          const int nbid = t.nbr[(size_t)id * 27 + 13 + (side ? w[d] : -w[d])];
+          if (nbid == -1) continue;               // outside the domain
           if (nbid >= n) {                        // refined neighbour: this leaf is coarse
             coarse_side = true;
             t.refl[id].coarse_mask |= 1 << (2 * d + side);
@@ -559,35 +603,6 @@ namespace mapgb {
 
 namespace {
 
-// leaf index (pool id < nleaves) covering block (p, L, c) of the current tree: the block
-// itself, or the leaf at a coarser level that contains it; -1 if the block region is
-// refined below L (then no single leaf covers it) or outside the domain.
-int covering_leaf(const HostTree& t, int p, int L, const int* c) {
-  int ijk[3] = {c[0], c[1], c[2]};
-  for (int l = L; l >= 0; --l) {
-    const int id = t.find(p, l, ijk[0], ijk[1], ijk[2]);
-    if (id >= 0) return id < t.nleaves ? id : -1;
-    for (int d = 0; d < 3; ++d) ijk[d] >>= 1;
-  }
-  return -1;
-}
-
-// neighbour block coordinates of (p, L, c) in direction off, periodic wrap; false if the
-// neighbour lies outside a non-periodic boundary
-bool neighbour(const std::vector<map_problem_desc>& probs, int ndim, int p, int L, const int* c, const int* off,
-               int* q) {
-  for (int d = 0; d < 3; ++d) q[d] = c[d];
-  for (int d = 0; d < ndim; ++d) {
-    const int n = probs[p].nbase[d] << L;
-    q[d] = c[d] + off[d];
-    if (q[d] < 0 || q[d] >= n) {
-      if (probs[p].bc[d][q[d] < 0 ? 0 : 1] != MAP_BC_PERIODIC) return false;
-      q[d] = (q[d] + n) % n;
-    }
-  }
-  return true;
-}
-
 template <typename F>
 void for_each_offset(int ndim, F&& f) {
   for (int oz = (ndim == 3 ? -1 : 0); oz <= (ndim == 3 ? 1 : 0); ++oz)
@@ -607,7 +622,7 @@ void for_each_offset(int ndim, F&& f) {
 // when the coarsened parent keeps the 2:1 rule.  New leaves are listed in the order of the
 // old leaves: a kept leaf in place, a refined leaf as its 2^ndim children (child bits
 // x | y<<1 | z<<2 ascending), a coarsened parent at the place of its first child.
-std::string plan_regrid(const HostTree& t, const std::vector<map_problem_desc>& probs, const int8_t* flags,
+std::string plan_regrid(const HostTree& t, const int8_t* flags,
                         int max_level, std::vector<map_block_desc>& out) {
   const int n = t.nleaves, nd = t.ndim;
   out.clear();
@@ -624,18 +639,14 @@ std::string plan_regrid(const HostTree& t, const std::vector<map_problem_desc>& 
   while (!work.empty()) {
     const int id = work.back();
     work.pop_back();
-    const int p = t.blk_problem[id], L = t.blk_level[id];
-    const int* c = &t.blk_ijk[3 * id];
     for_each_offset(nd, [&](const int* off) {
-      int q[3];
-      if (!neighbour(probs, nd, p, L, c, off, q)) return;
-      const int cov = covering_leaf(t, p, L, q);
-      if (cov < 0 || refine[cov]) return;
-      if (t.blk_level[cov] < L) {
-        if (t.blk_level[cov] >= max_level) return;  // cannot happen in a balanced tree
-        refine[cov] = 1;
-        work.push_back(cov);
-      }
+      // a coarser neighbour, which becomes as fine as this leaf
+      const int at = t.nbr[(size_t)id * 27 + (off[0] + 1) + 3 * (off[1] + 1) + 9 * (off[2] + 1)];
+      if (at > -2) return;
+      const int cov = -2 - at;
+      if (refine[cov] || t.blk_level[cov] >= max_level) return;
+      refine[cov] = 1;
+      work.push_back(cov);
     });
   }
   // coarsening candidates: parents whose children are all leaves flagged -1, none refined
@@ -657,15 +668,18 @@ std::string plan_regrid(const HostTree& t, const std::vector<map_problem_desc>& 
     changed = false;
     for (int par = n; par < t.nblocks; ++par) {
       if (!coarsen[par]) continue;
-      const int p = t.blk_problem[par], L = t.blk_level[par] + 1;   // children level
-      const int* c = &t.blk_ijk[3 * par];
       bool bad = false;
       for_each_offset(nd, [&](const int* off) {
         if (bad) return;
-        int q[3];
-        if (!neighbour(probs, nd, p, L - 1, c, off, q)) return;
-        const int nb = t.find(p, L - 1, q[0], q[1], q[2]);
-        if (nb < 0 || nb < n) return;                 // coarser or a leaf at L-1: fine
+        // the block of the parent's level in that direction: the parent of what lies beyond the
+        // child on that side
+        int side = 0;
+        for (int d = 0; d < nd; ++d)
+          if (off[d] == 1) side |= 1 << d;
+        const int ch0 = t.children[(size_t)par * 8 + side];
+        const int at = t.nbr[(size_t)ch0 * 27 + (off[0] + 1) + 3 * (off[1] + 1) + 9 * (off[2] + 1)];
+        if (at < 0) return;                           // outside, or a leaf at L-1: fine
+        const int nb = t.parent[at];
         // neighbour parent at L-1: its children touching us must end at level <= L
         if (coarsen[nb]) return;
         for (int cb = 0; cb < (1 << nd); ++cb) {
@@ -687,12 +701,12 @@ std::string plan_regrid(const HostTree& t, const std::vector<map_problem_desc>& 
     }
   }
   std::vector<char> emitted(t.nblocks, 0);
+  out.reserve(n);
   for (int l = 0; l < n; ++l) {
     const int id = t.leaf_to_block[l];
     const int p = t.blk_problem[id], L = t.blk_level[id];
     const int* c = &t.blk_ijk[3 * id];
-    int par = -1;
-    if (L > 0) par = t.find(p, L - 1, c[0] >> 1, c[1] >> 1, c[2] >> 1);
+    const int par = t.parent[id];
     if (par >= 0 && coarsen[par]) {
       if (!emitted[par]) {
         emitted[par] = 1;
