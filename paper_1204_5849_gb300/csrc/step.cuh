@@ -673,9 +673,9 @@ step_kernel(StepArgsT<T> A) {
               T a[NV], b[NV], fa[NV], fb[NV];
 #pragma unroll
               for (int v = 0; v < NV; ++v) {
-                T ph = limiter<T, LIM>(w[v] - plm[v * P2 + cm], plp[v * P2 + cp] - w[v]);
-                a[v] = w[v] + T(0.5) * ph;
-                b[v] = w[v] - T(0.5) * ph;
+                const T ph = half_limiter<T, LIM>(w[v] - plm[v * P2 + cm], plp[v * P2 + cp] - w[v]);
+                a[v] = w[v] + ph;
+                b[v] = w[v] - ph;
               }
               flux_p<T, D>(a, pressure<T>(a, P), P, fa);
               flux_p<T, D>(b, pressure<T>(b, P), P, fb);
@@ -747,10 +747,8 @@ step_kernel(StepArgsT<T> A) {
           const T um = up[v * P2 + cl - st], u1 = up[v * P2 + cl];
           const T u2 = up[v * P2 + cl + st], u3 = up[v * P2 + cl + 2 * st];
           if (SCHEME == SCH_LF) {
-            T phl = limiter<T, LIM>(u1 - um, u2 - u1);
-            T phr = limiter<T, LIM>(u2 - u1, u3 - u2);
-            a[v] = tp[v * RING + rl] + T(0.5) * phl;
-            b[v] = tp[v * RING + rl + rs] - T(0.5) * phr;
+            a[v] = tp[v * RING + rl] + half_limiter<T, LIM>(u1 - um, u2 - u1);
+            b[v] = tp[v * RING + rl + rs] - half_limiter<T, LIM>(u2 - u1, u3 - u2);
           } else {
             a[v] = weno_minus_right<T>(um, u1, u2);
             b[v] = weno_plus_left<T>(u1, u2, u3);
@@ -835,10 +833,8 @@ step_kernel(StepArgsT<T> A) {
         for (int v = 0; v < NV; ++v) {
           const T um = um1[v], u1 = p0[v * P2 + cown], u2 = p1[v * P2 + cown], u3 = p2[v * P2 + cown];
           if (SCHEME == SCH_LF) {
-            T phl = limiter<T, LIM>(u1 - um, u2 - u1);
-            T phr = limiter<T, LIM>(u2 - u1, u3 - u2);
-            a[v] = tslot(z)[v * RING + rown] + T(0.5) * phl;
-            b[v] = tslot(z + 1)[v * RING + rown] - T(0.5) * phr;
+            a[v] = tslot(z)[v * RING + rown] + half_limiter<T, LIM>(u1 - um, u2 - u1);
+            b[v] = tslot(z + 1)[v * RING + rown] - half_limiter<T, LIM>(u2 - u1, u3 - u2);
           } else {
             a[v] = weno_minus_right<T>(um, u1, u2);
             b[v] = weno_plus_left<T>(u1, u2, u3);
