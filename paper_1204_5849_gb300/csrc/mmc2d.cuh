@@ -79,20 +79,6 @@ __device__ __forceinline__ void flux_pairs_of(const float* q, const Comps& w, fl
   c.e = q[FEN];
 }
 
-// minmod as max(min(a, b), 0) + min(max(a, b), 0): the smaller magnitude where the signs agree,
-// else 0 (five operations without predicates; a NaN on one side gives the other side's value
-// or 0, and the state that made it is NaN in the face's flux itself)
-template <int LIM>
-__device__ __forceinline__ float limit(float a, float b) {
-  if (LIM != 0) return limiter<float, LIM>(a, b);
-  return fmaxf(fminf(a, b), 0.0f) + fminf(fmaxf(a, b), 0.0f);
-}
-template <int LIM>
-__device__ __forceinline__ float2 limit2(float2 a, float2 b) {
-  if (LIM != 0) return pair::limiter2<LIM>(a, b);
-  return make_float2(limit<LIM>(a.x, b.x), limit<LIM>(a.y, b.y));
-}
-
 // 1. in FP32: two x-neighbours per thread, one in each lane of the paired operations; of the
 // outermost rows only the pairs over the interior columns are read
 template <int NB, int NT>
@@ -196,7 +182,7 @@ __device__ __forceinline__ float2 combine(float2 a, float2 b, float2 w0, float2 
   const float2 gmc = pair::sub(fm, pair::fma(nb, t0, g0));
   const float2 gpc = pair::sub(pair::fma(b, t1, g1), fp);
   const float2 gmr = pair::sub(pair::fma(na, w3, f3), pair::fma(nb, t1, g1));
-  const float2 l = pair::sub(limit2<LIM>(gpl, gpc), limit2<LIM>(gmr, gmc));
+  const float2 l = pair::sub(pair::limiter2<LIM>(gpl, gpc), pair::limiter2<LIM>(gmr, gmc));
   return pair::fma(pair::splat(0.25f), l, pair::mul(pair::splat(0.5f), pair::add(fp, fm)));
 }
 
@@ -432,7 +418,7 @@ __device__ __forceinline__ void faces_f32(const float* su, const float* st, cons
       const float gmc = fm - (g[e0].e - b * t[e0].e);
       const float gpc = (g[e1].e + b * t[e1].e) - fp;
       const float gmr = (f[c3].e - a * w[c3].e) - (g[e1].e - b * t[e1].e);
-      F[EN] = 0.5f * (fp + fm) + 0.25f * (limit<LIM>(gpl, gpc) - limit<LIM>(gmr, gmc));
+      F[EN] = 0.5f * (fp + fm) + 0.25f * (limiter<float, LIM>(gpl, gpc) - limiter<float, LIM>(gmr, gmc));
     }
 #pragma unroll
     for (int v = 0; v < NV; ++v) dst[var_of(yd, v) * NFACE + k * ds] = F[v];
