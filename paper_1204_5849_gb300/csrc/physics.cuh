@@ -600,5 +600,62 @@ __device__ __forceinline__ void lf_flux2(const float2* ab, const Phys<float>& P,
   }
 }
 
+// MMC in FP32 with the states of a stencil in the lanes (3D; 2D has mmc2d.cuh).
+//
+// The predictor's flux difference along D, h_{i+1/2} - h_{i-1/2}, times two: the cells i-1 and
+// i+1 in the lanes of ab, w and a0 the cell's own state and speed.  Its own flux cancels, and
+// the dissipation is taken on differences.
+template <int D, bool OOL>
+__device__ __forceinline__ void mmc_diff2(const float2* ab, const float* w, float a0, const Phys<float>& P, float* g) {
+  float2 f[NV], al;
+  flux2<D, OOL>(ab, P, f, &al);
+  const float2 na = make_float2(-fmaxf(al.x, a0), -fmaxf(a0, al.y));
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const float2 s = glm_pair<D>(v) ? splat(-P.ch) : na;
+    const float2 r = fma(s, sub(ab[v], splat(w[v])), make_float2(-f[v].x, f[v].y));
+    g[v] = r.x + r.y;
+  }
+}
+
+// The face between cells i and i+1: load_c fills the lanes with u_i, u_{i+1}, load_o with
+// u_{i-1}, u_{i+2}, load_t with u~_i, u~_{i+1}; the split fluxes of mmc_face, doubled (the limiters
+// scale).  Six scalar fluxes and pressures and four speeds become three, three and two paired
+// ones.  Each pair is loaded when its turn comes, so that only split fluxes are held across the
+// next pair's.  Four steps of 112x80x96 (210 16^3 blocks) with the state in and out: 950 us with
+// scalar fluxes, 863 with mmc_diff2, 799 with both.
+template <int D, int LIM, bool OOL, typename LC, typename LO, typename LT>
+__device__ __forceinline__ void mmc_face2(const Phys<float>& P, float* F, LC load_c, LO load_o, LT load_t) {
+  float2 sc[NV], so[NV], x[NV], f[NV], al;
+  load_c(x);
+  flux2<D, OOL>(x, P, f, &al);
+  const float alpha = fmaxf(al.x, al.y);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const float a = glm_pair<D>(v) ? P.ch : alpha;
+    sc[v] = fma(make_float2(a, -a), x[v], f[v]);                // f+_i, f-_{i+1}
+  }
+  load_o(x);
+  flux2<D, OOL>(x, P, f, nullptr);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const float a = glm_pair<D>(v) ? P.ch : alpha;
+    so[v] = fma(make_float2(a, -a), x[v], f[v]);                // f+_{i-1}, f-_{i+2}
+  }
+  load_t(x);
+  flux2<D, OOL>(x, P, f, &al);
+  const float alphat = fmaxf(al.x, al.y);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const float b = glm_pair<D>(v) ? P.ch : alphat;
+    const float2 tp = fma(splat(b), x[v], f[v]);                // f~+_i, f~+_{i+1}
+    const float2 tm = fma(splat(-b), x[v], f[v]);               // f~-_i, f~-_{i+1}
+    const float2 gp = sub(tp, make_float2(so[v].x, sc[v].x));   // g+_{i-1/2}, g+_{i+1/2}
+    const float2 gm = sub(make_float2(sc[v].y, so[v].y), tm);   // g-_{i+1/2}, g-_{i+3/2}
+    F[v] = 0.5f * (sc[v].x + sc[v].y) +
+           0.25f * (limiter<float, LIM>(gp.x, gp.y) - limiter<float, LIM>(gm.y, gm.x));
+  }
+}
+
 }  // namespace pair
 }  // namespace mapgb

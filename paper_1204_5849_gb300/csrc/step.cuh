@@ -622,6 +622,23 @@ step_kernel(StepArgsT<T> A) {
           else mmc2d::predict<T, NB>(ul[1], sr, c, lam, P, acc);
 #pragma unroll
           for (int v = 0; v < NV; ++v) tp[v * RING + r] = acc[v];
+        } else if constexpr (SCHEME == SCH_MMC && std::is_same<T, float>::value) {
+          const T pw = pressure<T>(w, P);
+          auto dir = [&](auto Dc, const T* plm, int cm, const T* plp, int cp) {
+            constexpr int D = decltype(Dc)::value;
+            float2 ab[NV];
+            T g[NV];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) ab[v] = make_float2(plm[v * P2 + cm], plp[v * P2 + cp]);
+            pair::mmc_diff2<D, true>(ab, w, alpha_p<T, D>(w, pw, P), P, g);
+#pragma unroll
+            for (int v = 0; v < NV; ++v) acc[v] -= lamh[D] * g[v];
+          };
+          dir(std::integral_constant<int, 0>(), ul[1], c - 1, ul[1], c + 1);
+          dir(std::integral_constant<int, 1>(), ul[1], c - NP, ul[1], c + NP);
+          dir(std::integral_constant<int, 2>(), ul[0], c, ul[2], c);
+#pragma unroll
+          for (int v = 0; v < NV; ++v) tp[v * RING + r] = acc[v];
         } else if (SCHEME == SCH_MMC) {
           T wm[NV], wp[NV], hp[NV], hm[NV];
           ldw<T, P2>(ul[1], c - 1, wm);
@@ -712,7 +729,16 @@ step_kernel(StepArgsT<T> A) {
     // with the same operations on the same operands, so both directions share one instance
     // of the flux code (and a warp may hold faces of both)
     auto face_xy = [&](bool yd, const T* up, const T* tp, int cl, int st, int rl, int rs, T* F) {
-      if (SCHEME == SCH_MMC) {
+      if constexpr (SCHEME == SCH_MMC && std::is_same<T, float>::value) {
+        auto ends = [&](const T* a, int S, int i0, int i1, float2* x) {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) x[v] = make_float2(a[v * S + i0], a[v * S + i1]);
+          exch_xy(yd, x);
+        };
+        pair::mmc_face2<0, LIM, true>(P, F, [&](float2* x) { ends(up, P2, cl, cl + st, x); },
+                                          [&](float2* x) { ends(up, P2, cl - st, cl + 2 * st, x); },
+                                          [&](float2* x) { ends(tp, RING, rl, rl + rs, x); });
+      } else if (SCHEME == SCH_MMC) {
         T w0[NV], w1[NV], w2[NV], w3[NV], t0[NV], t1[NV];
         ldw<T, P2>(up, cl - st, w0);
         ldw<T, P2>(up, cl, w1);
@@ -805,7 +831,18 @@ step_kernel(StepArgsT<T> A) {
       const T* p0 = uslot(z);
       const T* p1 = uslot(z + 1);
       const T* p2 = uslot(z + 2);
-      if (SCHEME == SCH_MMC) {
+      if constexpr (SCHEME == SCH_MMC && std::is_same<T, float>::value) {
+        auto ends = [&](const T* a, const T* b, int S, int i, float2* x) {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) x[v] = make_float2(a[v * S + i], b[v * S + i]);
+        };
+        pair::mmc_face2<2, LIM, true>(P, F, [&](float2* x) { ends(p0, p1, P2, cown, x); },
+                                          [&](float2* x) {
+#pragma unroll
+                                            for (int v = 0; v < NV; ++v) x[v] = make_float2(um1[v], p2[v * P2 + cown]);
+                                          },
+                                          [&](float2* x) { ends(tslot(z), tslot(z + 1), RING, rown, x); });
+      } else if (SCHEME == SCH_MMC) {
         T w1[NV], w2[NV], w3[NV], t0[NV], t1[NV];
         ldw<T, P2>(p0, cown, w1);
         ldw<T, P2>(p1, cown, w2);
