@@ -118,7 +118,7 @@ typedef struct {
   int subcycle;       /* 1: n = ceil(dt/dt_c) conduction substeps of dt/n inside each step,
                          dt_c = c_cfl min(dx)^2 / (n_dim max(kappa/rho)); 0: dt <= dt_c and
                          one update.  With conduction, map_advance reads dt back every step
-                         to size the loop and is not graph-replayed */
+                         to size the loop */
   double grad_t_max;  /* > 0: face temperature gradients clipped to +-grad_t_max (Sec. 3.6
                          threshold); 0: none */
 } map_params;
@@ -247,7 +247,7 @@ int map_last_sums(map_pool* pool, double* sums_out);
 /* Launch shape chosen by map_autotune. */
 typedef struct {
   int grid;           /* step-kernel CTAs: 0 = the default (one per block in 3D; for FP32
-                         pools in 2D a persistent grid of four per SM), a value >= the
+                         pools in 2D a persistent grid of the resident CTAs, 3 to 8 per SM), a value >= the
                          block count = one per block, else a persistent grid */
   int w_pred, w_face; /* warp-schedule cost of a predictor unit and of a face unit */
   double ms_default;  /* step launches with the default shape (grid 0, default
@@ -348,7 +348,7 @@ int map_get_speeds_async(map_pool* pool, double* out);
 int map_get_speeds(map_pool* pool, double* out);
 
 /* (No counterpart in the paper.)  Number of kernels the library launched since the pool
- * was created (graph replays count each kernel in the graph). */
+ * was created (replayed graphs of conduction substeps count each kernel in them). */
 long long map_kernel_launches(const map_pool* pool);
 
 /* Last error text of the pool (or of the last failed create when pool is NULL). */

@@ -772,12 +772,15 @@ int map_cfl_dt(map_pool* pool, const map_params* p, double* dt_out) {
 }
 
 // Grid of the FP32 single step launch: the tuned one, else one CTA per block in 3D and, in
-// 2D (256-cell blocks, whose per-block reductions weigh), a persistent grid of as many CTAs
-// per SM as the 128-thread 2D FP32 kernels have resident: three for MMC, else four.
+// 2D (64- and 256-cell blocks, whose per-block reductions weigh), a persistent grid of as many
+// CTAs per SM as the kernel has resident: three of 16^2 and six of 8^2 for MMC, else four and
+// eight.  (4096 8^2 blocks, six steps, on four per SM against these: LF 319 -> 235 us, WENO 469 ->
+// 344, MMC 353 -> 285; eight per SM for MMC 350.)
 static int step_grid(const map_pool* pool, const map_params* p) {
   if (pool->tune_grid > 0) return pool->tune_grid;
-  if (!is64(pool) && pool->ndim == 2 && pool->nsm > 0) return (p->scheme == MAP_MMC && pool->nb == 16 ? 3 : 4) * pool->nsm;
-  return 0;
+  if (is64(pool) || pool->ndim != 2 || pool->nsm <= 0) return 0;
+  const int resident = (p->scheme == MAP_MMC ? 3 : 4) * (pool->nb == 8 ? 2 : 1);
+  return resident * pool->nsm;
 }
 
 // The block list of the FP32 single launch with grid G: for a persistent grid, the leaves
