@@ -504,6 +504,26 @@ __device__ __forceinline__ float2 limiter2(float2 a, float2 b) {
   return make_float2(pr.x > 0.0f ? __fdividef(q.x, s.x) : 0.0f, pr.y > 0.0f ? __fdividef(q.y, s.y) : 0.0f);
 }
 
+// The limited slopes as the MUSCL-Hancock states take them: slope2 times SLOPE_HALF is half the
+// slope.  van Leer's ab/(a+b) is the half already (its factor of two cancels exactly), minmod
+// keeps its half for the multiply-add that builds the states.  (256^3, four steps: 8626 -> 8541
+// us.)
+template <int LIM>
+constexpr float SLOPE_HALF = LIM ? 1.0f : 0.5f;
+template <int LIM>
+__device__ __forceinline__ float2 slope2(float2 a, float2 b) {
+  if (LIM == 0) return limiter2<LIM>(a, b);
+  const float2 pr = mul(a, b);
+  const float2 s = add(a, b);
+  return make_float2(pr.x > 0.0f ? __fdividef(pr.x, s.x) : 0.0f, pr.y > 0.0f ? __fdividef(pr.y, s.y) : 0.0f);
+}
+template <int LIM>
+__device__ __forceinline__ float slope(float a, float b) {
+  if (LIM == 0) return limiter<float, LIM>(a, b);
+  const float pr = a * b;
+  return pr > 0.0f ? __fdividef(pr, a + b) : 0.0f;
+}
+
 // pressure of two states (same FP64 fallback rule as pressure<float>); OOL: the FP64
 // recovery out of line (as pressure<float> has it) or inline, whichever measures faster in
 // the calling kernel (inline in the 3D 16^3 kernels, which sit at their register cap)

@@ -669,19 +669,20 @@ step_kernel(StepArgsT<T> A) {
             if constexpr (std::is_same<T, float>::value) {
               // the two half-states u +- phi/2 in the lanes of a float2
               float2 ab[NV], fab[NV];
+              const float2 half2 = make_float2(pair::SLOPE_HALF<LIM>, -pair::SLOPE_HALF<LIM>);
               // the limited slopes of two variables at a time
 #pragma unroll
               for (int v = 0; v + 1 < NV; v += 2) {
                 const float2 wv = make_float2(w[v], w[v + 1]);
                 const float2 lo = make_float2(plm[v * P2 + cm], plm[(v + 1) * P2 + cm]);
                 const float2 hi = make_float2(plp[v * P2 + cp], plp[(v + 1) * P2 + cp]);
-                const float2 ph = pair::limiter2<LIM>(pair::sub(wv, lo), pair::sub(hi, wv));
-                ab[v] = pair::fma(pair::splat(ph.x), make_float2(0.5f, -0.5f), pair::splat(w[v]));
-                ab[v + 1] = pair::fma(pair::splat(ph.y), make_float2(0.5f, -0.5f), pair::splat(w[v + 1]));
+                const float2 ph = pair::slope2<LIM>(pair::sub(wv, lo), pair::sub(hi, wv));
+                ab[v] = pair::fma(pair::splat(ph.x), half2, pair::splat(w[v]));
+                ab[v + 1] = pair::fma(pair::splat(ph.y), half2, pair::splat(w[v + 1]));
               }
               {
-                const T ph = limiter<T, LIM>(w[NV - 1] - plm[(NV - 1) * P2 + cm], plp[(NV - 1) * P2 + cp] - w[NV - 1]);
-                ab[NV - 1] = pair::fma(pair::splat(ph), make_float2(0.5f, -0.5f), pair::splat(w[NV - 1]));
+                const T ph = pair::slope<LIM>(w[NV - 1] - plm[(NV - 1) * P2 + cm], plp[(NV - 1) * P2 + cp] - w[NV - 1]);
+                ab[NV - 1] = pair::fma(pair::splat(ph), half2, pair::splat(w[NV - 1]));
               }
               pair::flux2<D, !(NDIM == 3 && NB == 16)>(ab, P, fab, nullptr);
 #pragma unroll
@@ -760,9 +761,9 @@ step_kernel(StepArgsT<T> A) {
           const float2 ulo = make_float2(up[v * P2 + cl - st], up[v * P2 + cl]);      // (u_i-1, u_i)
           const float2 umid = make_float2(up[v * P2 + cl], up[v * P2 + cl + st]);    // (u_i, u_i+1)
           const float2 uhi = make_float2(up[v * P2 + cl + st], up[v * P2 + cl + 2 * st]);
-          const float2 ph = pair::limiter2<LIM>(pair::sub(umid, ulo), pair::sub(uhi, umid));
+          const float2 ph = pair::slope2<LIM>(pair::sub(umid, ulo), pair::sub(uhi, umid));
           const float2 tt = make_float2(tp[v * RING + rl], tp[v * RING + rl + rs]);
-          ab[v] = pair::fma(ph, make_float2(0.5f, -0.5f), tt);
+          ab[v] = pair::fma(ph, make_float2(pair::SLOPE_HALF<LIM>, -pair::SLOPE_HALF<LIM>), tt);
         }
         exch_xy(yd, ab);
         pair::lf_flux2<0, !(NDIM == 3 && NB == 16)>(ab, *reinterpret_cast<const Phys<float>*>(&P), reinterpret_cast<float*>(F), (float)kc[16]);
@@ -859,9 +860,9 @@ step_kernel(StepArgsT<T> A) {
           const float2 ulo = make_float2(um1[v], p0[v * P2 + cown]);
           const float2 umid = make_float2(p0[v * P2 + cown], p1[v * P2 + cown]);
           const float2 uhi = make_float2(p1[v * P2 + cown], p2[v * P2 + cown]);
-          const float2 ph = pair::limiter2<LIM>(pair::sub(umid, ulo), pair::sub(uhi, umid));
+          const float2 ph = pair::slope2<LIM>(pair::sub(umid, ulo), pair::sub(uhi, umid));
           const float2 tt = make_float2(t0p[v * RING + rown], t1p[v * RING + rown]);
-          ab[v] = pair::fma(ph, make_float2(0.5f, -0.5f), tt);
+          ab[v] = pair::fma(ph, make_float2(pair::SLOPE_HALF<LIM>, -pair::SLOPE_HALF<LIM>), tt);
         }
         pair::lf_flux2<2, !(NDIM == 3 && NB == 16)>(ab, *reinterpret_cast<const Phys<float>*>(&P), reinterpret_cast<float*>(F), (float)kc[16]);
       } else {
