@@ -53,3 +53,26 @@ def test_loop_equals_per_substep_path(gpulib, geom, mode, prec):
         assert len(set(int(q) for q in counts[0])) > 1, counts[0]      # the problems differ in substeps
     assert int(counts[0].max()) > 1
     np.testing.assert_array_equal(out[0], out[1])
+
+
+def test_loops_of_several_pools_at_once(gpulib):
+    """Three pools on streams of their own, each with more leaves than SMs: their substep loops
+    are enqueued without waiting for one another and give what one pool alone gives."""
+    from paper_1204_5849_gb300 import MAP_FP32_FIX64, Pool
+    mesh = w.uniform_mesh(2, 16, (16, 16))
+    U0 = _state(mesh)
+    p = dict(gamma=5 / 3, c_cfl=0.4, scheme="lf", limiter="minmod", conduction="aligned", kappa0=3.0 / 256, subcycle=1)
+    pools = [Pool(mesh, MAP_FP32_FIX64) for _ in range(3)]
+    for q in pools:
+        q.write_leaves(U0)
+    for _ in range(6):
+        for q in pools:
+            q.advance(p, 1)
+    assert [q.check() for q in pools] == [0, 0, 0]
+    ref = Pool(mesh, MAP_FP32_FIX64)
+    ref.write_leaves(U0)
+    ref.set_conduction_loop(False)
+    ref.advance(p, 6)
+    want = ref.read_leaves()
+    for q in pools:
+        np.testing.assert_array_equal(q.read_leaves(), want)

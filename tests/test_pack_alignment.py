@@ -14,13 +14,18 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("ndim,nb,nbase", [(2, 8, (3, 5, 1)), (2, 16, (5, 2, 1)), (3, 8, (2, 3, 1)), (3, 16, (1, 2, 1))])
 @pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("shift", [0, 1, 2])
-def test_pack_and_unpack_at_any_element_offset(gpulib, ndim, nb, nbase, prec, shift):
+@pytest.mark.parametrize("order", ["forward", "reversed", "part"])
+def test_pack_and_unpack_at_any_element_offset(gpulib, ndim, nb, nbase, prec, shift, order):
     import torch
     from paper_1204_5849_gb300 import Pool
     mesh = w.uniform_mesh(ndim, nb, nbase)
     dt = torch.float64 if prec == 0 else torch.float32
-    ids = np.arange(mesh.nleaves, dtype=np.int32)[::-1].copy()     # any order of leaves
-    shape = (mesh.nleaves, 9) + mesh.block_shape()
+    ids = np.arange(mesh.nleaves, dtype=np.int32)                  # the whole state in leaf order
+    if order == "reversed":
+        ids = ids[::-1].copy()
+    elif order == "part":
+        ids = ids[1:].copy()
+    shape = (len(ids), 9) + mesh.block_shape()
     n = int(np.prod(shape))
     g = torch.Generator().manual_seed(1204 + shift)
     src = torch.empty(n + 4, dtype=dt, device="cuda")
