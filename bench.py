@@ -431,8 +431,8 @@ def main():
     clocks.start()
     barrier()
     l0 = pool.kernel_launches()
-    # one event before every step and one after the last: the per-step intervals time the
-    # graph replay of each step (finalize, a 72-byte memset and the step kernel)
+    # one event before every step and one after the last: the per-step intervals time each
+    # step's launches (finalize and the step kernel)
     evs = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps + 1)]
     evs[0].record(stream)
     for i in range(args.steps):
@@ -479,7 +479,7 @@ def main():
         return
 
     # -------- the interface fluxes on the same workload (Sec. 3.2-3.3, Sec. 5): the step with
-    # HLLC and with HLLD in place of f_m, graph-replayed like the value (untimed by the line's
+    # HLLC and with HLLD in place of f_m (untimed by the line's
     # value; the state moves on, and the end-to-end loop below writes its own) --------------
     riemann_ms = {"f_m": ms / args.steps}
     nr = min(args.steps, 20)
@@ -642,7 +642,7 @@ def main():
         "warmup": args.warmup, "ms_per_step": ms_max / args.steps, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": WORKLOAD, "cells": ncells, "blocks": mesh.nleaves,
-                   "block": "16^3 + 2 ghost layers", "form": "fp32+fp64-fix batched, graph-replayed",
+                   "block": "16^3 + 2 ghost layers", "form": "fp32+fp64-fix batched",
                    "l2": "state (1.2 GB) larger than L2; no flush",
                    "launch_shape": tune,
                    "parallelism": f"replicas x{world}" if world > 1 else "1 GPU"},

@@ -29,7 +29,7 @@ def choose_block_size(make_mesh: Callable[[int], object], make_state: Callable[[
         try:
             pool.write_leaves(make_state(mesh))
             shape = pool.autotune(params, reps=reps)
-            pool.advance(params, 1)                      # capture the step graph
+            pool.advance(params, 1)                      # the first step also sets kernel attributes
             pool.check()
             t0 = time.perf_counter()
             pool.advance(params, steps)

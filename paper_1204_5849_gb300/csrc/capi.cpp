@@ -1190,11 +1190,11 @@ int map_advance(map_pool* pool, const map_params* p, int nsteps) {
     if (rc) return rc;
     pool->alpha_ready = true;
   }
-  // Plain launches: a step is two of them on a uniform mesh, up to twenty on a refined one, and the host
-  // enqueues a launch in about 2.5 us, faster than the device runs it, while a step replayed as
-  // one CUDA graph left 4 to 5 us between two graphs, across which no launch overlapped the
-  // kernel before it.  Per pass, a graph per step -> this: 128^2 MMC, ten steps 218 -> 174 us;
-  // 720x528 HLLC, four steps 262 -> 250; 112x80x96 MMC 1004 -> 990; 2992-leaf rotor (17
+  // Plain launches: a step is two of them on a uniform mesh, up to twenty on a refined one, and
+  // the host enqueues a launch in about 2.5 us, faster than the device runs it, while a step
+  // replayed as one CUDA graph left 4 to 5 us between two graphs, across which no launch
+  // overlapped the kernel before it.  Per pass, a graph per step -> this: 128^2 MMC, ten steps 218
+  // -> 174 us; 720x528 HLLC, four steps 262 -> 250; 112x80x96 MMC 1004 -> 990; 2992-leaf rotor (17
   // launches a step) 848 -> 844; 9472-leaf octree 4645 -> 4643.
   for (int s = 0; s < nsteps; ++s) {
     rc = advance_once(pool, p);
