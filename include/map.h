@@ -156,7 +156,8 @@ int map_set_stream(map_pool* pool, void* stream);
  * another, every parent complete, 2:1 balance across faces, edges and corners) and builds
  * the neighbour / ghost-fill tables on the host.  Leaf data is undefined until written.
  * Leaf index l of later calls is the position in this array.  Errors: MAP_EINVAL,
- * MAP_ENOMEM (more blocks than max_blocks). */
+ * MAP_ENOMEM (more blocks than max_blocks): the tree set before stays.  MAP_ECUDA (no device
+ * memory for the tables): the pool has no tree until map_set_tree succeeds. */
 int map_set_tree(map_pool* pool, const map_block_desc* leaves, int n);
 
 /* Copy one leaf's interior from / to the host (FP64 [9][nz][nb][nb]).  read synchronises. */
@@ -211,7 +212,7 @@ int map_flag_refine(map_pool* pool, const map_params* p, const map_refine_params
  * or a parent of old leaves).  Kept leaves copy, new children are prolonged from their
  * old parent (Sec. 4.3 formula on the interior), new parents take the restriction of
  * their old children.  Ghosts of the old tree must be filled.  Leaf indices follow the
- * new array.  Errors: MAP_EINVAL. */
+ * new array.  Errors: as map_set_tree (which then restores a pool without a tree). */
 int map_regrid(map_pool* pool, const map_block_desc* new_leaves, int n);
 
 /* Regrid decision on the host (Sec. 4.5 "refine if the error exceeds the threshold"):

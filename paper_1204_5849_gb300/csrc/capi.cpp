@@ -349,7 +349,10 @@ int map_set_stream(map_pool* pool, void* stream) {
   return MAP_OK;
 }
 
+// Until it succeeds the pool has no tree: the tables are written in place, so a call that ran
+// after an allocation failed half way would address the new ones with the old tree's numbers.
 static int install_tree(map_pool* pool, HostTree& t) {
+  pool->have_tree = false;
   forget_tree(pool);
   drop_graphs(pool);
   pool->cond_copies = -1;
@@ -364,8 +367,8 @@ static int install_tree(map_pool* pool, HostTree& t) {
   CK(D.refl.upload(t.refl, pool->stream));
   if (!t.reflux_tasks.empty()) {
     CK(D.rtasks.upload(t.reflux_tasks, pool->stream));
-    D.nrtasks = (int)t.reflux_tasks.size();
     CK(D.freg.reserve((size_t)t.nslots * 2 * pool->ndim * kNV * pool->nb * pool->nb * pool->elem));
+    D.nrtasks = (int)t.reflux_tasks.size();
   }
   std::vector<int> ll, pl, rl;
   D.leaf_off.assign(t.maxlev + 2, 0);
@@ -405,12 +408,16 @@ static int install_tree(map_pool* pool, HostTree& t) {
   if (need > pool->staging_elems) {
     cudaFree(pool->staging);
     pool->staging = nullptr;
+    pool->staging_elems = 0;
     CK(cudaMalloc(&pool->staging, need * sizeof(double)));
     pool->staging_elems = need;
   }
   if (t.nleaves > pool->flags_cap) {
     cudaFree(pool->flags);
     cudaFree(pool->est);
+    pool->flags = nullptr;
+    pool->est = nullptr;
+    pool->flags_cap = 0;
     CK(cudaMalloc(&pool->flags, t.nleaves));
     CK(cudaMalloc(&pool->est, t.nleaves * sizeof(double)));
     pool->flags_cap = t.nleaves;
@@ -1256,6 +1263,7 @@ int map_regrid(map_pool* pool, const map_block_desc* leaves, int n) {
   if ((int)tasks.size() > pool->tasks_cap) {
     cudaFree(pool->tasks);
     pool->tasks = nullptr;
+    pool->tasks_cap = 0;
     CK(cudaMalloc(&pool->tasks, tasks.size() * sizeof(RegridTask)));
     pool->tasks_cap = (int)tasks.size();
   }

@@ -1,0 +1,124 @@
+"""The device memory a pool holds, without a GPU: the C ABI (capi.cpp, tree.cpp) built against
+tests/host/host_runtime.cpp, whose allocations are host memory that can be made to run out and
+whose launchers check that every table they are given reaches to its last entry."""
+
+from __future__ import annotations
+
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import workloads as w
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+PARAMS = dict(gamma=5 / 3, c_cfl=0.4, scheme="lf", limiter="minmod")
+
+
+@pytest.fixture(scope="module")
+def hostlib(tmp_path_factory):
+    from paper_1204_5849_gb300 import _build, binding
+    try:
+        cuda = _build._cuda_home(_build._nvcc())
+    except RuntimeError as e:
+        pytest.skip(str(e))
+    out = str(tmp_path_factory.mktemp("hostlib") / "libhost.so")
+    # (-Bsymbolic: the library keeps its own runtime where the process has loaded another)
+    cmd = ["g++", "-O1", "-std=c++17", "-fPIC", "-shared", "-pthread", "-Wl,-Bsymbolic", "-I", _build.INCLUDE,
+           "-I", os.path.join(cuda, "include"), os.path.join(_build.CSRC, "capi.cpp"),
+           os.path.join(_build.CSRC, "tree.cpp"), os.path.join(HERE, "host", "host_runtime.cpp"), "-o", out]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    lib = C.CDLL(out)
+    for name, (res, args) in binding._SIGS.items():
+        fn = getattr(lib, name)
+        fn.restype, fn.argtypes = res, args
+    lib.host_fail_from.argtypes = [C.c_longlong]
+    return lib
+
+
+@pytest.fixture
+def host(hostlib, monkeypatch):
+    from paper_1204_5849_gb300 import binding
+    monkeypatch.setattr(binding, "_lib", hostlib)
+    hostlib.host_fail_from(0)
+    yield hostlib
+    hostlib.host_fail_from(0)
+
+
+def counts(lib):
+    v = (C.c_longlong * 6)()
+    lib.host_counts(v)
+    return dict(zip(("bytes", "launches", "bad", "syncs", "d2h", "graphs"), (int(x) for x in v)))
+
+
+def _small():
+    return w.uniform_mesh(2, 8, (4, 4), lo=(-0.5, -0.5, 0), hi=(0.5, 0.5, 1))
+
+
+def _amr(levels=2):
+    return w.radial_amr_mesh(2, 8, (4, 4), levels, radii=(0.12, 0.45)[2 - levels:], bc=w.mesh.PERIODIC)
+
+
+def _use(pool, mesh):
+    """Every call that walks the tree's tables."""
+    pool.write_leaves(np.ones((mesh.nleaves,) + pool.interior_shape()))
+    pool.advance(PARAMS, 3)
+    pool.fill_ghosts()
+    pool.cfl_dt(PARAMS)
+    pool.step(PARAMS)
+    pool.flag_refine(PARAMS, dict(thr=0.2))
+    pool.conservation()
+    pool.read_leaves()
+    pool.read_block(0)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("how", ["set_tree", "regrid"])
+def test_a_tree_that_does_not_fit_leaves_no_tree(host, prec, how):
+    """Memory that runs out anywhere while a larger tree is installed: the call fails, no later
+    call launches a kernel on tables of two trees, and a tree that fits is taken again."""
+    from paper_1204_5849_gb300 import MapError, Pool
+    small, big = _small(), _amr(1)
+    failed = 0
+    for k in range(1, 40):
+        pool = Pool(small, prec, max_blocks=400)
+        host.host_set_blocks(400)
+        _use(pool, small)
+        host.host_fail_from(k)
+        try:
+            getattr(pool, how)(big)
+        except MapError:
+            failed += 1
+            host.host_fail_from(0)
+            before = counts(host)
+            taken = []
+            for call in (lambda: pool.fill_ghosts(), lambda: pool.cfl_dt(PARAMS), lambda: pool.advance(PARAMS, 2),
+                         lambda: pool.conservation(), lambda: pool.read_block(0)):
+                try:
+                    call()
+                    taken.append(True)
+                except MapError as e:
+                    taken.append(e.code != -8)               # MAP_ESTATE
+            after = counts(host)
+            assert after["bad"] == before["bad"], (k, taken)
+            # either the old tree still stands whole, or there is none
+            assert len(set(taken)) == 1, (k, taken)
+            if not taken[0]:
+                assert after["launches"] == before["launches"], k
+            for mesh in (small, big):
+                pool.set_tree(mesh)
+                _use(pool, mesh)
+            assert counts(host)["bad"] == before["bad"], k
+            pool.close()
+            assert counts(host)["bad"] == before["bad"], k
+        else:
+            host.host_fail_from(0)
+            _use(pool, big)
+            pool.close()
+            assert counts(host)["bad"] == 0
+            break
+    assert failed >= 5
+    assert counts(host)["bytes"] == 0
