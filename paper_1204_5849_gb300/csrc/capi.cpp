@@ -509,6 +509,7 @@ static int write_leaves_async(map_pool* pool, const void* u, int f32) {
   if (need > pool->astaging_elems) {
     CK(cudaStreamSynchronize(pool->copy_stream));
     CK(cudaStreamSynchronize(pool->stream));
+    pool->astaging_elems = 0;
     for (int k = 0; k < 2; ++k) {
       cudaFree(pool->astaging[k]);
       pool->astaging[k] = nullptr;
@@ -556,6 +557,7 @@ static int read_leaves_async(map_pool* pool, void* u, int f32) {
   if (bytes > pool->rstaging_bytes) {
     CK(cudaStreamSynchronize(pool->rcopy_stream));
     CK(cudaStreamSynchronize(pool->stream));
+    pool->rstaging_bytes = 0;
     for (int k = 0; k < 2; ++k) {
       cudaFree(pool->rstaging[k]);
       pool->rstaging[k] = nullptr;

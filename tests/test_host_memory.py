@@ -122,3 +122,27 @@ def test_a_tree_that_does_not_fit_leaves_no_tree(host, prec, how):
             break
     assert failed >= 5
     assert counts(host)["bytes"] == 0
+
+
+@pytest.mark.parametrize("how", ["write_leaves_async_ptr", "read_leaves_async_ptr", "read_leaves_async_f32_ptr"])
+def test_staging_that_does_not_fit_is_not_used(host, how):
+    """Memory that runs out while the staging buffers of the asynchronous copies grow: a later
+    copy of a smaller tree takes new buffers, not the ones given back."""
+    from paper_1204_5849_gb300 import MapError, Pool
+    small, big = _small(), _amr(1)
+    U = np.ones((big.nleaves, 9) + big.block_shape())
+    for k in (1, 2):
+        pool = Pool(small, 1, max_blocks=400)
+        host.host_set_blocks(400)
+        getattr(pool, how)(U.ctypes.data)
+        pool.set_tree(big)
+        host.host_fail_from(k)
+        with pytest.raises(MapError):
+            getattr(pool, how)(U.ctypes.data)
+        host.host_fail_from(0)
+        pool.set_tree(small)
+        before = counts(host)["bad"]
+        getattr(pool, how)(U.ctypes.data)
+        getattr(pool, how)(U.ctypes.data)
+        pool.close()
+        assert counts(host)["bad"] == before
