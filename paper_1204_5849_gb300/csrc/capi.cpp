@@ -11,14 +11,15 @@
 
 using namespace mapgb;
 
-// A device array that is kept from tree to tree and grown when a larger one needs it.
+// A device array that is kept from tree to tree: grown, with a quarter to spare, when a larger
+// tree needs it, and given back when a tree needs less than half of it (4 KB aside).
 template <typename X>
 struct DevArray {
   X* p = nullptr;
   size_t cap = 0;
   operator X*() const { return p; }
   cudaError_t reserve(size_t n) {
-    if (n <= cap) return cudaSuccess;
+    if (n <= cap && cap * sizeof(X) <= 2 * n * sizeof(X) + 4096) return cudaSuccess;
     release();
     const size_t want = n + n / 4;
     cudaError_t e = cudaMalloc((void**)&p, want * sizeof(X));
@@ -369,6 +370,9 @@ static int install_tree(map_pool* pool, HostTree& t) {
     CK(D.rtasks.upload(t.reflux_tasks, pool->stream));
     CK(D.freg.reserve((size_t)t.nslots * 2 * pool->ndim * kNV * pool->nb * pool->nb * pool->elem));
     D.nrtasks = (int)t.reflux_tasks.size();
+  } else {
+    D.rtasks.release();
+    D.freg.release();
   }
   std::vector<int> ll, pl, rl;
   D.leaf_off.assign(t.maxlev + 2, 0);
