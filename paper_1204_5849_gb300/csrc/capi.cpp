@@ -66,11 +66,16 @@ struct DevTree {
   std::vector<int> act_off;    // offsets per level (host)
   int n_act = 0;
   int* xfer_ids = nullptr;     // pool ids of the leaves of one map_pack_leaves / map_unpack_leaves
-  // the FP32 single launch's block list for a persistent grid of chunk_grid CTAs: CTA c's
-  // grid-stride positions c, c + G, ... hold a contiguous Morton range of the leaves
-  int* chunk_ids = nullptr;
-  int chunk_grid = 0;
-  bool chunk_partial = false;
+  std::vector<int> act_ids;    // act_all (host)
+  // the FP32 single launch's block lists for persistent grids: with a grid of `grid` CTAs, CTA
+  // c's grid-stride positions c, c + grid, ... hold a contiguous Morton range of the (active)
+  // leaves.  Two of them: the default grids of MMC and of the other schemes differ
+  struct ChunkList {
+    int* ids = nullptr;
+    int grid = 0;              // 0: not built for the present tree and active leaves
+  };
+  ChunkList chunks[2];
+  int chunk_next = 0;
 };
 
 struct map_pool {
@@ -188,10 +193,12 @@ static void forget_tree(map_pool* pool) {
   cudaFree(D.act_all);
   cudaFree(D.act_level);
   cudaFree(D.xfer_ids);
-  cudaFree(D.chunk_ids);
-  D.act_all = D.act_level = D.xfer_ids = D.chunk_ids = nullptr;
-  D.n_act = D.nrtasks = D.chunk_grid = 0;
-  D.chunk_partial = false;
+  for (auto& c : D.chunks) {
+    cudaFree(c.ids);
+    c = DevTree::ChunkList();
+  }
+  D.act_all = D.act_level = D.xfer_ids = nullptr;
+  D.n_act = D.nrtasks = 0;
   pool->partial = false;
 }
 
@@ -799,35 +806,38 @@ static int step_grid(const map_pool* pool, const map_params* p) {
 // The block list of the FP32 single launch with grid G: for a persistent grid, the leaves
 // (or the active ones) reordered so that each CTA's grid-stride positions hold one contiguous
 // Morton range (its blocks then share problem and level in long runs, over which the kernel
-// reduces its fused diagnostics once).  Built outside stream capture; during a capture
-// without it the plain order is used.
+// reduces its fused diagnostics once).  Built outside stream capture, once per tree (or active
+// set) and grid, two grids being kept; during a capture without it the plain order is used.
 static int step_block_list(map_pool* pool, int G, const int** list) {
   DevTree& D = pool->dt;
   const HostTree& t = pool->tree;
   const int n = pool->partial ? D.n_act : t.nleaves;
   *list = pool->partial ? D.act_all : D.all_leaves.p;
   if (G <= 0 || G >= n) return MAP_OK;
-  if (D.chunk_ids && D.chunk_grid == G && D.chunk_partial == pool->partial) {
-    *list = D.chunk_ids;
-    return MAP_OK;
-  }
+  for (const auto& c : D.chunks)
+    if (c.grid == G) {
+      *list = c.ids;
+      return MAP_OK;
+    }
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(pool->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return MAP_OK;
-  std::vector<int> src(n), perm(n);
-  CK(cudaMemcpyAsync(src.data(), *list, (size_t)n * sizeof(int), cudaMemcpyDeviceToHost, pool->stream));
-  CK(cudaStreamSynchronize(pool->stream));
+  const std::vector<int>& src = pool->partial ? D.act_ids : t.all_leaves;
+  std::vector<int> perm(n);
   int start = 0;
   for (int c = 0; c < G; ++c) {
     const int len = c < n ? (n - 1 - c) / G + 1 : 0;   // positions c, c + G, ... below n
     for (int k = 0; k < len; ++k) perm[c + (size_t)k * G] = src[start + k];
     start += len;
   }
-  if (!D.chunk_ids) CK(cudaMalloc(&D.chunk_ids, (size_t)t.nleaves * sizeof(int)));
-  CK(cudaMemcpyAsync(D.chunk_ids, perm.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice, pool->stream));
-  CK(cudaStreamSynchronize(pool->stream));
-  D.chunk_grid = G;
-  D.chunk_partial = pool->partial;
-  *list = D.chunk_ids;
+  DevTree::ChunkList& c = D.chunks[D.chunk_next];
+  D.chunk_next ^= 1;
+  c.grid = 0;
+  if (!c.ids) CK(cudaMalloc(&c.ids, (size_t)t.nleaves * sizeof(int)));
+  // (stream-ordered behind the steps that read the list before)
+  CK(cudaMemcpyAsync(c.ids, perm.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice, pool->stream));
+  CK(cudaStreamSynchronize(pool->stream));             // the host list goes out of scope
+  c.grid = G;
+  *list = c.ids;
   return MAP_OK;
 }
 
@@ -1621,7 +1631,7 @@ int map_set_active(map_pool* pool, const int* leaves, int n) {
   cudaFree(D.act_level);
   D.act_all = D.act_level = nullptr;
   D.n_act = 0;
-  D.chunk_grid = 0;
+  for (auto& c : D.chunks) c.grid = 0;
   pool->partial = false;
   drop_graphs(pool);
   pool->have_dt = false;
@@ -1650,6 +1660,7 @@ int map_set_active(map_pool* pool, const int* leaves, int n) {
   }
   CK(cudaStreamSynchronize(pool->stream));
   D.n_act = (int)all.size();
+  D.act_ids.swap(all);
   pool->partial = true;
   return MAP_OK;
 }

@@ -177,3 +177,39 @@ def test_a_pool_that_has_coarsened_gives_its_memory_back(host, prec):
         _use(pool, mesh)
     pool.close()
     assert counts(host)["bad"] == 0 and counts(host)["bytes"] == 0
+
+
+def test_schemes_that_alternate_keep_their_block_lists(host):
+    """A 2D FP32 pool whose steps alternate between schemes (persistent grids of two sizes): the
+    reordered block lists are built once per tree and grid, without waiting for the stream, and
+    again after the active leaves or the tree change."""
+    from paper_1204_5849_gb300 import Pool
+    mesh = w.uniform_mesh(2, 8, (12, 12))                   # 144 blocks, grids of 24 and 32 CTAs
+    pool = Pool(mesh, 1, max_blocks=400)
+    host.host_set_blocks(400)
+    schemes = ("mmc", "lf", "weno")
+
+    def waits(n):
+        c0 = counts(host)
+        for _ in range(n):
+            for s in schemes:
+                pool.advance(dict(PARAMS, scheme=s), 1)
+        c1 = counts(host)
+        assert c1["bad"] == 0
+        assert c1["d2h"] == c0["d2h"]                       # no ids are read back
+        return c1["syncs"] - c0["syncs"]
+
+    assert waits(1) <= 2                                    # one wait per list
+    assert waits(5) == 0
+    pool.set_active(np.arange(100, dtype=np.int32))
+    for s in ("mmc", "lf"):
+        pool.cfl_dt(dict(PARAMS, scheme=s))
+        pool.step(dict(PARAMS, scheme=s))
+    pool.set_active(None)
+    assert waits(1) <= 2
+    assert waits(5) == 0
+    pool.set_tree(mesh)
+    assert waits(1) <= 2
+    assert waits(5) == 0
+    pool.close()
+    assert counts(host)["bad"] == 0 and counts(host)["bytes"] == 0
