@@ -152,7 +152,7 @@ __device__ __forceinline__ void predict(const float* su, const float* R, int c, 
     flux(-st, wm, fm);
     flux(st, wp, fp);
     const float a0 = Rd[SPD * P2];
-    const float am = fmaxf(Rd[SPD * P2 - st], a0), ap = fmaxf(a0, Rd[SPD * P2 + st]);
+    const float am = dmax(Rd[SPD * P2 - st], a0), ap = dmax(a0, Rd[SPD * P2 + st]);
     const float hl = -0.5f * lam[d];
     auto upd = [&](int k, float sm, float sp, float& o0, float& o1) {
       float2 g = pair::sub(fp.p[k], fm.p[k]);
@@ -171,6 +171,24 @@ __device__ __forceinline__ void predict(const float* su, const float* R, int c, 
   }
 }
 
+// FP32 minmod as max(min(a, b), 0) + min(max(a, b), 0), the inner two handing a NaN on (a gradient
+// without a value limits to 0, as minmod_lim's): one operation more on the ALU pipe than
+// minmod_lim, one of the five on the FMA pipe, and faster in this walk (32640 16^2 blocks, four
+// steps: 3819 us against 3858)
+template <int LIM>
+__device__ __forceinline__ float limit(float a, float b) {
+  if (LIM != 0) return limiter<float, LIM>(a, b);
+  float lo, hi;
+  asm("min.ftz.NaN.f32 %0, %1, %2;" : "=f"(lo) : "f"(a), "f"(b));
+  asm("max.ftz.NaN.f32 %0, %1, %2;" : "=f"(hi) : "f"(a), "f"(b));
+  return fmaxf(lo, 0.0f) + fminf(hi, 0.0f);
+}
+template <int LIM>
+__device__ __forceinline__ float2 limit2(float2 a, float2 b) {
+  if (LIM != 0) return pair::limiter2<LIM>(a, b);
+  return make_float2(limit<LIM>(a.x, b.x), limit<LIM>(a.y, b.y));
+}
+
 // one component (pair) of a face: twice the split fluxes (the limiters scale), the halves in
 // the last two factors
 template <int LIM>
@@ -182,7 +200,7 @@ __device__ __forceinline__ float2 combine(float2 a, float2 b, float2 w0, float2 
   const float2 gmc = pair::sub(fm, pair::fma(nb, t0, g0));
   const float2 gpc = pair::sub(pair::fma(b, t1, g1), fp);
   const float2 gmr = pair::sub(pair::fma(na, w3, f3), pair::fma(nb, t1, g1));
-  const float2 l = pair::sub(pair::limiter2<LIM>(gpl, gpc), pair::limiter2<LIM>(gmr, gmc));
+  const float2 l = pair::sub(limit2<LIM>(gpl, gpc), limit2<LIM>(gmr, gmc));
   return pair::fma(pair::splat(0.25f), l, pair::mul(pair::splat(0.5f), pair::add(fp, fm)));
 }
 
@@ -399,7 +417,8 @@ __device__ __forceinline__ void faces_f32(const float* su, const float* st, cons
     const int c0 = k & 3, c1 = (k + 1) & 3, c2 = (k + 2) & 3, c3 = (k + 3) & 3, e0 = k & 1, e1 = e0 ^ 1;
     load_u(k + 3, w[c3], f[c3], al[c3]);
     load_t(k + 1, t[e1], g[e1], at[e1]);
-    const float a = fmaxf(al[c1], al[c2]), b = fmaxf(at[e0], at[e1]);
+    // (a face whose u~ has no speed on its right takes the first-order flux: its gradients are NaN)
+    const float a = dmax(al[c1], al[c2]), b = dmax(at[e0], at[e1]);
     float F[NV];
     auto comb = [&](int p, float sa, float sb, float& o0, float& o1) {
       const float2 x = combine<LIM>(pair::splat(sa), pair::splat(sb), w[c0].p[p], w[c1].p[p], w[c2].p[p], w[c3].p[p],
@@ -418,7 +437,7 @@ __device__ __forceinline__ void faces_f32(const float* su, const float* st, cons
       const float gmc = fm - (g[e0].e - b * t[e0].e);
       const float gpc = (g[e1].e + b * t[e1].e) - fp;
       const float gmr = (f[c3].e - a * w[c3].e) - (g[e1].e - b * t[e1].e);
-      F[EN] = 0.5f * (fp + fm) + 0.25f * (limiter<float, LIM>(gpl, gpc) - limiter<float, LIM>(gmr, gmc));
+      F[EN] = 0.5f * (fp + fm) + 0.25f * (limit<LIM>(gpl, gpc) - limit<LIM>(gmr, gmc));
     }
 #pragma unroll
     for (int v = 0; v < NV; ++v) dst[var_of(yd, v) * NFACE + k * ds] = F[v];

@@ -30,7 +30,7 @@ struct Phys {
 };
 
 template <typename T>
-__device__ __forceinline__ T dmax(T a, T b) { return a > b ? a : b; }
+__device__ __forceinline__ T dmax(T a, T b) { return a > b ? a : b; }   // keeps a NaN on its right
 
 // a / b.  FP64: the plain quotient (rounds as the same formula written in plain C).  FP32:
 // the fast quotient, reciprocal times numerator (within 2 ulp); every FP32 quotient on the
@@ -425,12 +425,16 @@ __device__ __forceinline__ bool positive<double>(double x) {
   return (unsigned long long)(__double_as_longlong(x) - 1) < 0x7ff0000000000000ull;
 }
 
-// minmod in FP32 as max(min(a, b), 0) + min(max(a, b), 0): four min/max and an addition in place
-// of a minimum, four comparisons and two selects, which all share the half-rate ALU pipe.  The
-// values are minmod's (a zero's sign aside); where one side is NaN it gives the other side's
-// value or 0 in place of 0, and the cell that holds the NaN is NaN in its own flux.
+// minmod in FP32: the smaller magnitude with the product's sign in one minimum, cut at 0, with a's
+// sign -- three operations in place of a minimum, four comparisons and two selects, which all
+// share the half-rate ALU pipe.  The minimum hands a NaN on and the cut takes 0 in its place, so
+// the values are minmod's for every input (a zero's sign aside): a gradient without a value limits
+// to 0.  (9472-leaf octree, four steps: 4270 us with max(min(a, b), 0) + min(max(a, b), 0) and the
+// same NaN rule -> 4071.)
 __device__ __forceinline__ float minmod_lim(float a, float b) {
-  return fmaxf(fminf(a, b), 0.0f) + fminf(fmaxf(a, b), 0.0f);
+  float m;
+  asm("min.ftz.NaN.xorsign.abs.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
+  return copysignf(fmaxf(m, 0.0f), a);
 }
 __device__ __forceinline__ double minmod_lim(double a, double b) { return minmod<double>(a, b); }
 
@@ -629,7 +633,7 @@ template <int D, bool OOL>
 __device__ __forceinline__ void mmc_diff2(const float2* ab, const float* w, float a0, const Phys<float>& P, float* g) {
   float2 f[NV], al;
   flux2<D, OOL>(ab, P, f, &al);
-  const float2 na = make_float2(-fmaxf(al.x, a0), -fmaxf(a0, al.y));
+  const float2 na = make_float2(-dmax(al.x, a0), -dmax(a0, al.y));
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     const float2 s = glm_pair<D>(v) ? splat(-P.ch) : na;
@@ -649,7 +653,7 @@ __device__ __forceinline__ void mmc_face2(const Phys<float>& P, float* F, LC loa
   float2 sc[NV], so[NV], x[NV], f[NV], al;
   load_c(x);
   flux2<D, OOL>(x, P, f, &al);
-  const float alpha = fmaxf(al.x, al.y);
+  const float alpha = dmax(al.x, al.y);
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     const float a = glm_pair<D>(v) ? P.ch : alpha;
@@ -664,7 +668,7 @@ __device__ __forceinline__ void mmc_face2(const Phys<float>& P, float* F, LC loa
   }
   load_t(x);
   flux2<D, OOL>(x, P, f, &al);
-  const float alphat = fmaxf(al.x, al.y);
+  const float alphat = dmax(al.x, al.y);
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     const float b = glm_pair<D>(v) ? P.ch : alphat;
