@@ -12,15 +12,19 @@
 using namespace mapgb;
 
 // A device array that is kept from tree to tree: grown, with a quarter to spare, when a larger
-// tree needs it, and given back when a tree needs less than half of it (4 KB aside).
+// tree needs it, and given back when a tree needs less than half of it and leaves over kKeep
+// bytes unused (below that a pool that goes to and fro between two trees would allocate at every
+// regrid, 56 us in 193 of a small quadtree's two regrids).
 template <typename X>
 struct DevArray {
+  static constexpr size_t kKeep = 256 << 10;
   X* p = nullptr;
   size_t cap = 0;
   operator X*() const { return p; }
   cudaError_t reserve(size_t n) {
-    if (n <= cap && cap * sizeof(X) <= 2 * n * sizeof(X) + 4096) return cudaSuccess;
+    if (n <= cap && (cap <= 2 * n || (cap - n) * sizeof(X) <= kKeep)) return cudaSuccess;
     release();
+    if (n == 0) return cudaSuccess;
     const size_t want = n + n / 4;
     cudaError_t e = cudaMalloc((void**)&p, want * sizeof(X));
     if (e != cudaSuccess) {             // no room to spare: the size itself
@@ -378,8 +382,8 @@ static int install_tree(map_pool* pool, HostTree& t) {
     CK(D.freg.reserve((size_t)t.nslots * 2 * pool->ndim * kNV * pool->nb * pool->nb * pool->elem));
     D.nrtasks = (int)t.reflux_tasks.size();
   } else {
-    D.rtasks.release();
-    D.freg.release();
+    CK(D.rtasks.reserve(0));
+    CK(D.freg.reserve(0));
   }
   std::vector<int> ll, pl, rl;
   D.leaf_off.assign(t.maxlev + 2, 0);

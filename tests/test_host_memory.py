@@ -152,29 +152,49 @@ def test_staging_that_does_not_fit_is_not_used(host, how):
 def test_a_pool_that_has_coarsened_gives_its_memory_back(host, prec):
     """One pool through trees that grow, shrink and grow again: every table fits its tree (the
     launches check it), and a small tree after a large one holds at most twice what the same tree
-    holds in a pool of its own (and 4 KB for each of the twelve tables), besides the copies' staging
-    and flags, which stay at the largest."""
+    holds in a pool of its own, and 256 KB for each of the twelve tables, besides the copies'
+    staging and flags, which stay at the largest."""
     from paper_1204_5849_gb300 import Pool
+    cap = 16000
 
     def held(mesh, fine):
         """Bytes of one pool with `mesh`, after `fine` where given."""
         base = counts(host)["bytes"]
-        pool = Pool(fine or mesh, prec, max_blocks=1200)
+        pool = Pool(fine or mesh, prec, max_blocks=cap)
         if fine:
             pool.set_tree(mesh)
         n = counts(host)["bytes"] - base
         pool.close()
         return n
 
-    host.host_set_blocks(1200)
-    fine, small = _amr(2), _small()
-    state = 3 * 1200 * 9 * 12 * 12 * (8 if prec == 0 else 4)          # the block pool itself
+    host.host_set_blocks(cap)
+    small = _small()
+    fine = w.radial_amr_mesh(2, 8, (4, 4), 5, radii=(0.25, 0.33, 0.4, 0.55, 0.9), bc=w.mesh.PERIODIC)
+    assert fine.nleaves > 3000
+    state = 3 * cap * 9 * 12 * 12 * (8 if prec == 0 else 4)           # the block pool itself
     kept = (fine.nleaves - small.nleaves) * (9 * 64 * 8 + 9)           # staging and flags
-    assert held(small, fine) - state - kept <= 2 * (held(small, None) - state) + 12 * 4096
-    pool = Pool(small, prec, max_blocks=1200)
-    for mesh in (small, _amr(1), fine, small, _amr(1), small, fine):
+    assert held(small, fine) - state - kept <= 2 * (held(small, None) - state) + 12 * (256 << 10)
+    pool = Pool(small, prec, max_blocks=cap)
+    for mesh in (small, _amr(1), fine, small, _amr(2), small, fine, _amr(1)):
         pool.set_tree(mesh)
         _use(pool, mesh)
+    pool.close()
+    assert counts(host)["bad"] == 0 and counts(host)["bytes"] == 0
+
+
+def test_a_pool_between_two_trees_allocates_nothing(host):
+    """A small tree that is refined and coarsened again by turns keeps its tables."""
+    from paper_1204_5849_gb300 import Pool
+    a, b = _small(), _amr(1)
+    pool = Pool(b, 1, max_blocks=400)
+    host.host_set_blocks(400)
+    for mesh in (a, b, a, b):
+        pool.set_tree(mesh)
+    host.host_fail_from(1)                                              # no allocation succeeds
+    for mesh in (a, b, a, b):
+        pool.set_tree(mesh)
+    host.host_fail_from(0)
+    _use(pool, b)
     pool.close()
     assert counts(host)["bad"] == 0 and counts(host)["bytes"] == 0
 
