@@ -33,11 +33,15 @@ template <typename T>
 __device__ __forceinline__ T dmax(T a, T b) { return a > b ? a : b; }   // keeps a NaN on its right
 
 // a / b.  FP64: the plain quotient (rounds as the same formula written in plain C).  FP32:
-// the fast quotient, reciprocal times numerator (within 2 ulp); every FP32 quotient on the
-// step path has a denominator (a density, a cell spacing, a sum of slopes, a WENO weight sum)
-// far below the 2^126 range where the fast form flushes to zero.  (HLLC and HLLD, a dozen
-// quotients a face: with the full-range quotient of a plain a / b four steps of a 720x528 mesh
-// took 161.5 us in place of 157.7.)
+// the fast quotient, reciprocal times numerator (within 2 ulp), which is 0 for a denominator
+// above 2^126.  The denominators it is used with on the step path are densities (whose reciprocal
+// the pressure and the speeds take the same way), cell spacings, sums of slopes, WENO weight sums,
+// speeds and differences of speeds (HLLC, HLLD), and in HLLD the mass fluxes rho (S - u) and
+// rho (S - u)(S - S_M) - B_m^2, which stay below it wherever the products of pressure and density
+// that HLLD forms are finite; in the conduction loop |B|^2, beside whose energy no finite
+// conductive flux counts at that size.  HLLC's contact speed and v* take the plain a / b.  (The plain
+// quotient everywhere in HLLC and HLLD, a dozen a face: four steps of a 720x528 mesh 161.5 us in
+// place of 157.7.)
 template <typename T>
 __device__ __forceinline__ T qdiv(T a, T b) { return a / b; }
 template <>
@@ -201,8 +205,10 @@ __device__ __forceinline__ void hllc_flux(const T* a, const T* b, const Phys<T>&
     for (int v = 0; v < NV; ++v) f[v] = F[1][v];
   } else {
     const T ra = w[0][RHO], rb = w[1][RHO];
-    const T sm = qdiv<T>(rb * u[1] * (sr - u[1]) - ra * u[0] * (sl - u[0]) - pt[1] + pt[0],
-                         rb * (sr - u[1]) - ra * (sl - u[0]));
+    // (the full-range quotient: both sides' mass fluxes and the star density can exceed 2^126
+    // where rho, p and the speeds do not)
+    const T sm = (rb * u[1] * (sr - u[1]) - ra * u[0] * (sl - u[0]) - pt[1] + pt[0]) /
+                 (rb * (sr - u[1]) - ra * (sl - u[0]));
     constexpr int T1 = D == 0 ? 1 : 0, T2 = D == 2 ? 1 : 2;   // tangential dimensions
     const T bt1 = qdiv<T>(sr * w[1][BX + T1] - sl * w[0][BX + T1] - (F[1][BX + T1] - F[0][BX + T1]), sr - sl);
     const T bt2 = qdiv<T>(sr * w[1][BX + T2] - sl * w[0][BX + T2] - (F[1][BX + T2] - F[0][BX + T2]), sr - sl);
@@ -225,8 +231,8 @@ __device__ __forceinline__ void hllc_flux(const T* a, const T* b, const Phys<T>&
     us[MX + T1] = rs * qdiv<T>(wk[MX + T1], wk[RHO]) - qdiv<T>(bm * (bt1 - wk[BX + T1]), ds);
     us[MX + T2] = rs * qdiv<T>(wk[MX + T2], wk[RHO]) - qdiv<T>(bm * (bt2 - wk[BX + T2]), ds);
     T vbs = sm * bm;
-    vbs += qdiv<T>(us[MX + T1], rs) * bt1;
-    vbs += qdiv<T>(us[MX + T2], rs) * bt2;
+    vbs += (us[MX + T1] / rs) * bt1;
+    vbs += (us[MX + T2] / rs) * bt2;
     us[BX + D] = bm;
     us[BX + T1] = bt1;
     us[BX + T2] = bt2;
