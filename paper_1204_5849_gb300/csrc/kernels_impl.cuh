@@ -12,11 +12,21 @@ cudaError_t launch_step_one(const StepLaunch& L, cudaStream_t s) {
   const bool res = L.eta > 0.0;
   const size_t smem = step_smem_bytes<T, NDIM, NB, SCHEME>(res);
   auto kern = step_kernel<T, NDIM, NB, SCHEME, LIM, STAGE, FLX, RFX>;
-  static bool attr_done[2] = {false, false};
-  if (!attr_done[res]) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the limit is the resistive form's for both (each form setting its own, an ideal step would
+  // lower it under a resistive one)
+  static bool attr_done = false;
+  if (!attr_done) {
+    size_t most = step_smem_bytes<T, NDIM, NB, SCHEME>(true);
+    int dev = 0, optin = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
     if (e != cudaSuccess) return e;
-    attr_done[res] = true;
+    if (optin > 0 && most + fa.sharedSizeBytes > (size_t)optin) most = step_smem_bytes<T, NDIM, NB, SCHEME>(false);
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    if (e != cudaSuccess) return e;
+    attr_done = true;
   }
   StepArgsT<T> A;
   A.u_in = (const T*)L.u_in;
