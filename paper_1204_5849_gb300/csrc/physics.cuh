@@ -428,7 +428,7 @@ template <typename T>
 __device__ __forceinline__ bool positive(T x) { return x > T(0); }
 template <>
 __device__ __forceinline__ bool positive<double>(double x) {
-  return (unsigned long long)(__double_as_longlong(x) - 1) < 0x7ff0000000000000ull;
+  return (unsigned long long)__double_as_longlong(x) - 1ull < 0x7ff0000000000000ull;
 }
 
 // minmod in FP32: the smaller magnitude with the product's sign in one minimum, cut at 0, with a's
