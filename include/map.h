@@ -192,8 +192,12 @@ int map_step(map_pool* pool, const map_params* p);
 /* nsteps x (ghost fill, dt on the device, step), asynchronous: the batched form.  The
  * step kernel also reduces alpha_g of the new state (the next dt) and the FP64
  * conservation sums of the new state, so a separate CFL pass runs only before the first
- * step after the state changed outside this call.  The steps are plain launches on the
- * pool's stream.  map_get_speeds reads the last dt. */
+ * step after the state changed outside this call.  The first steps after a change of the tree,
+ * the parameters or the launch settings are plain launches on the pool's stream; later ones of
+ * three launches and more are captured and replayed, four steps to a CUDA graph (the states are
+ * the same either way).  The call returns early unless it enqueues more than the driver queues
+ * for a stream, about a thousand launches or graphs: then it waits for room.  Under a capture of
+ * the stream by the caller every step is plain.  map_get_speeds reads the last dt. */
 int map_advance(map_pool* pool, const map_params* p, int nsteps);
 
 /* Device error word accumulated by the steps since the last check (rho <= 0, p < 0,
@@ -349,7 +353,7 @@ int map_get_speeds_async(map_pool* pool, double* out);
 int map_get_speeds(map_pool* pool, double* out);
 
 /* (No counterpart in the paper.)  Number of kernels the library launched since the pool
- * was created (replayed graphs of conduction substeps count each kernel in them). */
+ * was created (replayed graphs count each kernel in them). */
 long long map_kernel_launches(const map_pool* pool);
 
 /* Last error text of the pool (or of the last failed create when pool is NULL). */

@@ -161,6 +161,18 @@ struct map_pool {
   CondGraph cond_graph[8];
   int cond_next = 0;
   map_params cond_params{};
+  // steps of map_advance captured as graphs (replay_steps), for step_params: kGraphSteps steps and
+  // one step, per starting buffer q and fill kind (2q + 1: residual fill).  step_plain: plain steps
+  // since the last change of tree, parameters or launch settings; step_kernels: launches of one
+  // that follows another (0: none did yet)
+  struct StepGraph {
+    cudaGraphExec_t ex = nullptr;
+    long long kernels = 0;
+  };
+  StepGraph step_graph[2][4];
+  map_params step_params{};
+  int step_plain = 0;
+  long long step_kernels = 0;
 };
 
 static std::string g_create_error;
@@ -223,7 +235,18 @@ static void free_tree(map_pool* pool) {
   D.freg.release();
 }
 
+static void drop_step_graphs(map_pool* pool) {
+  for (auto& kind : pool->step_graph)
+    for (auto& g : kind) {
+      if (g.ex) cudaGraphExecDestroy(g.ex);
+      g = map_pool::StepGraph();
+    }
+  pool->step_plain = 0;
+  pool->step_kernels = 0;
+}
+
 static void drop_graphs(map_pool* pool) {
+  drop_step_graphs(pool);
   for (auto& c : pool->cond_graph) {
     if (c.ex) cudaGraphExecDestroy(c.ex);
     c = map_pool::CondGraph();
@@ -835,6 +858,7 @@ static int step_block_list(map_pool* pool, int G, const int** list) {
   }
   DevTree::ChunkList& c = D.chunks[D.chunk_next];
   D.chunk_next ^= 1;
+  if (c.grid) drop_step_graphs(pool);                  // captured steps may hold the list
   c.grid = 0;
   if (!c.ids) CK(cudaMalloc(&c.ids, (size_t)t.nleaves * sizeof(int)));
   // (stream-ordered behind the steps that read the list before)
@@ -1186,6 +1210,71 @@ static int advance_once(map_pool* pool, const map_params* p) {
   return step_launches(pool, p, true);
 }
 
+// Steps of map_advance as graphs.  A plain launch takes the host about 1.5 us and a graph 2 us
+// whatever it holds, so a program that drives several small pools from one thread, or takes
+// hundreds of steps in a call, waits for its own launches where a step has several; but between
+// two graphs the device idles for 4 to 5 us, across which no launch overlaps the kernel before it.
+// Hence four steps to a graph, and one only where a step is long enough to hide that.  Host time and
+// device time a step of one pool, and time a step of eight pools, in us (plain / one step to a
+// graph / four):
+//   64 16^2 leaves, uniform,     2 launches: 3.3 / 1.3 / 0.6, 14.0 / 18.6 / 14.5,  4.1 / 2.8 / 2.4
+//   25 16^2 leaves, outflow,     3 launches: 5.0 / 1.3 / 0.6, 16.3 / 18.6 / 16.1,  5.4 / 2.7 / 2.2
+//   100 16^2 leaves, 3 levels,   7 launches: 10.5 / 1.3 / 0.6, 33.5 / 35.1 / 32.6, 11.4 / 5.4 / 4.9
+//   512 8^3 leaves, 3 levels,    8 launches: 11.4 / 1.4 / 0.6, 93.5 / 90.4 / 90.5, 50.1 / 47.2 / 47.1
+//   100 16^2 leaves, 3 levels, WENO, 12:     17.5 / 1.4 / 0.6, 50.0 / 47.4 / 45.8, 18.8 / 7.7 / 7.4
+//   472 16^2 leaves, 4 levels, WENO, 18:     25.2 / 1.5 / 0.7, 82.0 / 80.1 / 78.1, 28.3 / 24.2 / 23.9
+// A capture takes 0.1 to 0.2 ms, so the first kPlainSteps steps after a change are plain (a run that
+// regrids every few steps stays so).
+static const int kGraphSteps = 4, kPlainSteps = 16;
+static const int kFourFrom = 3, kOneFrom = 8;      // launches a step from which either is taken
+
+// Enqueues n = kGraphSteps or 1 steps as one graph; false: nothing enqueued, take a plain step.
+static bool replay_steps(map_pool* pool, const map_params* p, int n) {
+  if (pool->step_plain < kPlainSteps || pool->step_kernels < (n > 1 ? kFourFrom : kOneFrom)) return false;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(pool->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;                                  // a caller's own capture takes plain launches
+  }
+  const int q = pool->cur;
+  map_pool::StepGraph& g = pool->step_graph[n > 1][2 * q + (pool->pushed[q] ? 1 : 0)];
+  if (!g.ex) {
+    if (cudaStreamBeginCapture(pool->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    const bool pushed0[3] = {pool->pushed[0], pool->pushed[1], pool->pushed[2]};
+    const long long before = pool->launches;
+    int rc = MAP_OK;
+    for (int s = 0; s < n && rc == MAP_OK; ++s) rc = advance_once(pool, p);
+    cudaGraph_t graph = nullptr;
+    const cudaError_t ce = cudaStreamEndCapture(pool->stream, &graph);
+    cudaGraphExec_t ex = nullptr;
+    if (rc == MAP_OK && ce == cudaSuccess && graph && cudaGraphInstantiate(&ex, graph, 0) == cudaSuccess) {
+      g.ex = ex;
+      g.kernels = pool->launches - before;
+    }
+    if (graph) cudaGraphDestroy(graph);
+    cudaGetLastError();
+    pool->cur = q;
+    for (int b = 0; b < 3; ++b) pool->pushed[b] = pushed0[b];
+    pool->launches = before;
+    if (!g.ex) {
+      pool->step_plain = 0;                        // try again later
+      return false;
+    }
+  }
+  if (cudaGraphLaunch(g.ex, pool->stream) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  pool->launches += g.kernels;
+  pool->pushed[1 - q] = true;
+  if (n > 1) pool->pushed[q] = true;
+  if (n & 1) pool->cur = 1 - q;
+  return true;
+}
+
 int map_advance(map_pool* pool, const map_params* p, int nsteps) {
   if (!pool) return MAP_EINVAL;
   int rc = check_params(pool, p);
@@ -1217,15 +1306,23 @@ int map_advance(map_pool* pool, const map_params* p, int nsteps) {
     if (rc) return rc;
     pool->alpha_ready = true;
   }
-  // Plain launches: a step is two of them on a uniform mesh, up to twenty on a refined one, and
-  // the host enqueues a launch in about 2.5 us, faster than the device runs it, while a step
-  // replayed as one CUDA graph left 4 to 5 us between two graphs, across which no launch
-  // overlapped the kernel before it.  Per pass, a graph per step -> this: 128^2 MMC, ten steps 218
-  // -> 174 us; 720x528 HLLC, four steps 262 -> 250; 112x80x96 MMC 1004 -> 990; 2992-leaf rotor (17
-  // launches a step) 848 -> 844; 9472-leaf octree 4645 -> 4643.
-  for (int s = 0; s < nsteps; ++s) {
+  if (!params_equal(pool->step_params, *p)) {
+    drop_step_graphs(pool);
+    pool->step_params = *p;
+  }
+  for (int s = 0; s < nsteps;) {
+    const int n = nsteps - s < kGraphSteps || pool->step_kernels < kFourFrom ? 1 : kGraphSteps;
+    if (replay_steps(pool, p, n)) {
+      s += n;
+      continue;
+    }
+    const bool steady = pool->pushed[pool->cur];
+    const long long before = pool->launches;
     rc = advance_once(pool, p);
     if (rc) return rc;
+    if (steady) pool->step_kernels = pool->launches - before;
+    ++pool->step_plain;
+    ++s;
   }
   pool->have_dt = false;
   pool->sums_valid = true;

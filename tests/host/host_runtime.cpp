@@ -54,7 +54,7 @@ int last_id(const int* ids, int n) {
 }
 
 cudaError_t launched(bool good, long long* cnt) {
-  ++launches;
+  if (!capturing) ++launches;
   if (cnt) ++*cnt;
   if (!good) ++bad;
   return cudaSuccess;
@@ -101,6 +101,8 @@ void host_fail_from(long long k) {
   fail_from = k;
   allocs = 0;
 }
+// a capture of the pool's stream by the caller, on or off
+void host_set_capturing(int on) { capturing = on != 0; }
 void host_set_blocks(int n) { pool_blocks = n; }
 // live device bytes, launches, launches that would have addressed memory outside their tables,
 // stream synchronisations, device-to-host copies, graph launches

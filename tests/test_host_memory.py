@@ -233,3 +233,74 @@ def test_schemes_that_alternate_keep_their_block_lists(host):
     assert waits(5) == 0
     pool.close()
     assert counts(host)["bad"] == 0 and counts(host)["bytes"] == 0
+
+
+def test_long_advances_do_not_wait_for_their_launches(host):
+    """map_advance on a refined mesh: after its first steps the host enqueues four steps at a time,
+    so several hundred of them fit the driver's queue; the count of kernels is that of plain steps.
+    A change of parameters, tree or launch settings starts anew, and a caller's capture holds plain
+    launches only."""
+    from paper_1204_5849_gb300 import Pool
+    mesh = _amr(2)
+    U = np.ones((mesh.nleaves, 9) + mesh.block_shape())
+    host.host_set_blocks(800)
+    p = dict(PARAMS, scheme="weno")
+    pool, plain = Pool(mesh, 1, max_blocks=800), Pool(mesh, 1, max_blocks=800)
+
+    def calls(n, **kw):
+        c0 = counts(host)
+        k0 = pool.kernel_launches()
+        pool.advance(dict(p, **kw), n)
+        c1 = counts(host)
+        assert c1["bad"] == 0
+        return c1["launches"] - c0["launches"], c1["graphs"] - c0["graphs"], pool.kernel_launches() - k0
+
+    def plain_kernels(n, **kw):
+        k0 = plain.kernel_launches()
+        for _ in range(n):
+            plain.set_launch()                                           # drops what is captured
+            plain.advance(dict(p, **kw), 1)
+        return plain.kernel_launches() - k0
+
+    for q in (pool, plain):
+        q.write_leaves(U)
+    assert calls(16)[1] == 0                                             # plain at first
+    per = plain_kernels(16) // 16
+    assert per >= 8
+    k = plain_kernels(300)
+    assert calls(300) == (0, 75, k)
+    assert calls(3) == (0, 3, plain_kernels(3))                          # one at a time
+    for q in (pool, plain):
+        q.write_leaves(U)                                                # every region is filled again
+    k = plain_kernels(9)                                                 # (with the first speeds' reduction)
+    got = calls(9)
+    assert got[1:] == (3, k) and got[0] == 2
+    assert calls(10, eta=1e-3)[1] == 0                                   # other parameters
+    plain_kernels(10, eta=1e-3)
+    pool.advance(p, 16)
+    pool.set_launch(3)
+    assert calls(8)[1] == 0
+    pool.set_launch()
+    pool.set_tree(mesh)
+    pool.write_leaves(U)
+    assert calls(16)[1] == 0
+    host.host_set_capturing(1)
+    assert calls(8)[1:] == (0, 8 * per)
+    host.host_set_capturing(0)
+    pool.close()
+    plain.close()
+    assert counts(host)["bad"] == 0 and counts(host)["bytes"] == 0
+
+
+def test_a_step_of_two_launches_stays_plain(host):
+    """... also where the first step of a call fills every ghost region, as after a host write."""
+    from paper_1204_5849_gb300 import Pool
+    mesh = w.uniform_mesh(2, 8, (4, 4))
+    host.host_set_blocks(400)
+    pool = Pool(mesh, 1, max_blocks=400)
+    c = counts(host)["graphs"]
+    for _ in range(5):
+        pool.write_leaves(np.ones((16, 9) + mesh.block_shape()))
+        pool.advance(PARAMS, 20)
+    assert counts(host)["graphs"] == c
+    pool.close()
