@@ -264,8 +264,8 @@ typedef struct {
 
 /* Autotuner (no counterpart in the paper): times this pool's step launches on its current
  * tree and state under candidate launch shapes -- the default, one CTA per block, or a
- * persistent grid of 1-16 x the SM count, then warp-schedule weight ratios from 1:1 to 6:1 for the per-plane
- * work list -- and keeps the
+ * persistent grid of 1-16 x the SM count, then warp-schedule weight ratios from 1:1 to 6:1 for
+ * the per-plane work list (not for 2D MMC, whose list holds units of one kind) -- and keeps the
  * fastest for later map_step / map_advance calls (results are bitwise the same under every
  * shape; the fused FP64 sums may differ in rounding).  The state is not changed: trials
  * write only the other buffers, and the step constants and sums are restored.  Ghosts are

@@ -1560,7 +1560,7 @@ int map_autotune(map_pool* pool, const map_params* p, int reps, map_tune_result*
   // weight ratios from 1:1 to 6:1 (only the ratio shapes the schedule); the default's is skipped
   const int W[][2] = {{1, 1}, {5, 4}, {3, 2}, {2, 1}, {9, 4}, {3, 1}, {4, 1}, {6, 1}};
   for (const auto& wgt : W) {
-    if (rc) break;
+    if (rc || (pool->ndim == 2 && p->scheme == MAP_MMC)) break;   // its schedule has units of one kind
     if (wgt[0] * dwf == wgt[1] * dwp) continue;
     rc = trial(bg, wgt[0], wgt[1], &t);
     if (rc == MAP_OK && t < best) { best = t; bwp = wgt[0]; bwf = wgt[1]; }

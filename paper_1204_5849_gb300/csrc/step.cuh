@@ -429,14 +429,15 @@ struct WorkList {
 // least-loaded warp that has room (ties to the lowest warp), a predictor unit weighing w_pred
 // and a face unit w_face (their relative cost; default_schedule_weights unless tuned).  s[w][15] holds the
 // number of units of warp w, s[w][0..] the units.  Without a predictor (WENO without
-// resistivity) its units are left out, so they do not displace face units.
+// resistivity) its units are left out, so they do not displace face units; 2D MMC's faces are not
+// in the list.
 template <int NDIM, int NB, int NT>
-inline void build_schedule(int w_pred, int w_face, bool pred, unsigned char (&s)[8][16]) {
+inline void build_schedule(int w_pred, int w_face, bool pred, bool faces, unsigned char (&s)[8][16]) {
   using W = WorkList<NDIM, NB, NT>;
   int load[8] = {0}, cnt[8] = {0};
   for (int q = 0; q < 8; ++q)
     for (int k = 0; k < 16; ++k) s[q][k] = 0;
-  for (int u = pred ? 0 : W::NPU; u < W::NU; ++u) {
+  for (int u = pred ? 0 : W::NPU; u < (faces ? W::NU : W::NPU); ++u) {
     int best = -1;
     for (int q = 0; q < W::NW; ++q)
       if (cnt[q] < 15 && (best < 0 || load[q] < load[best])) best = q;
@@ -730,7 +731,9 @@ step_kernel(StepArgsT<T> A) {
     // with the same operations on the same operands, so both directions share one instance
     // of the flux code (and a warp may hold faces of both)
     auto face_xy = [&](bool yd, const T* up, const T* tp, int cl, int st, int rl, int rs, T* F) {
-      if constexpr (SCHEME == SCH_MMC && std::is_same<T, float>::value) {
+      if constexpr (Mmc2d<NDIM, SCHEME>::value) {
+        // (mmc2d.cuh walks the faces)
+      } else if constexpr (SCHEME == SCH_MMC && std::is_same<T, float>::value) {
         auto ends = [&](const T* a, int S, int i0, int i1, float2* x) {
 #pragma unroll
           for (int v = 0; v < NV; ++v) x[v] = make_float2(a[v * S + i0], a[v * S + i1]);

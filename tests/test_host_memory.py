@@ -304,3 +304,22 @@ def test_a_step_of_two_launches_stays_plain(host):
         pool.advance(PARAMS, 20)
     assert counts(host)["graphs"] == c
     pool.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_autotune_leaves_the_weights_of_2d_mmc(host, prec):
+    """The schedule of 2D MMC holds units of one kind, which every weight shares out alike: the
+    tuner tries its grids only and keeps the default weights."""
+    from paper_1204_5849_gb300 import Pool
+    mesh = w.uniform_mesh(2, 8, (6, 6))
+    host.host_set_blocks(400)
+    tried = {}
+    for scheme in ("mmc", "lf"):
+        pool = Pool(mesh, prec, max_blocks=400)
+        pool.write_leaves(np.ones((36, 9) + mesh.block_shape()))
+        r = pool.autotune(dict(PARAMS, scheme=scheme), reps=1)
+        assert (r["w_pred"], r["w_face"]) == (7, 4)
+        tried[scheme] = r["trials"]
+        pool.close()
+    assert tried["lf"] - tried["mmc"] == 8                              # the weight ratios
+    assert counts(host)["bad"] == 0 and counts(host)["bytes"] == 0
