@@ -826,8 +826,7 @@ int map_cfl_dt(map_pool* pool, const map_params* p, double* dt_out) {
 static int step_grid(const map_pool* pool, const map_params* p) {
   if (pool->tune_grid > 0) return pool->tune_grid;
   if (is64(pool) || pool->ndim != 2 || pool->nsm <= 0) return 0;
-  const int resident = (p->scheme == MAP_MMC ? 3 : 4) * (pool->nb == 8 ? 2 : 1);
-  return resident * pool->nsm;
+  return step_resident_2d(pool->nb, p->scheme == MAP_MMC) * pool->nsm;
 }
 
 // The block list of the FP32 single launch with grid G: for a persistent grid, the leaves

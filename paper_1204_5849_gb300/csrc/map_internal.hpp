@@ -168,6 +168,13 @@ inline void default_schedule_weights(int ndim, int nb, int scheme, int* w_pred, 
   }
 }
 
+// CTAs per SM of the FP32 2D step kernels: the registers are bounded for so many (step_min_ctas),
+// shared memory lets them reside, and the default persistent grid holds them all (step_grid).
+// Four 128-thread 16^2 CTAs take the 128 registers two 256-thread ones did; 2D MMC's kept fluxes
+// (68 KB of shared memory for 16^2) let three reside, whose face walk then has 168 registers; an
+// 8^2 CTA is half of either.
+constexpr int step_resident_2d(int nb, bool mmc) { return (mmc ? 3 : 4) * (nb == 8 ? 2 : 1); }
+
 struct StepLaunch {
   const void* u_in;        // state with ghosts
   void* u_out;             // output state (interior written)

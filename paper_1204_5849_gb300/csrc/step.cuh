@@ -462,13 +462,10 @@ __device__ __forceinline__ void two_sum_acc(T& hi, T& lo, T h2, T l2) {
 // Without it none of that code exists in the kernel.
 // Resident CTAs per SM the register budget is sized for: the 3D 8^3 window (at most 36 KB of
 // shared memory) lets 6 CTAs reside, so asking for 8 would only cap the registers at 128 and
-// spill the column state; four 128-thread 2D 16^2 CTAs take the 128 registers two 256-thread
-// ones did.  2D MMC's kept fluxes (68 KB of shared memory for 16^2) let three reside, whose
-// face walk then has 168 registers.
+// spill the column state; 2D: step_resident_2d.
 template <typename T, int NDIM, int NB, int SCHEME>
 constexpr int step_min_ctas() {
-  return sizeof(T) != 4 ? 1 : NB == 16 ? (NDIM == 2 ? (Mmc2d<NDIM, SCHEME>::value ? 3 : 4) : 2)
-                                       : NDIM == 3 ? 6 : (Mmc2d<NDIM, SCHEME>::value ? 6 : 8);
+  return sizeof(T) != 4 ? 1 : NDIM == 2 ? step_resident_2d(NB, SCHEME == SCH_MMC) : NB == 16 ? 2 : 6;
 }
 
 template <typename T, int NDIM, int NB, int SCHEME, int LIM, int STAGE, int FLX, bool RFX>
