@@ -4,7 +4,7 @@ Workload: the 3D uniform linear Alfven wave, 256^3 cells as 4096 blocks of 16^3 
 layers), TVD-LF with the van Leer limiter, EGLM sources, gamma = 5/3 (synthetic input,
 closed-form initial condition).  A step is one pass of the whole hot path: ghost fill,
 CFL reduction (dt, c_h, c_p), the scheme update with sources and psi damping, and the FP64
-conservation sums.  `value` is the FP32 + FP64-fix batched form (graph-replayed
+conservation sums.  `value` is the FP32 + FP64-fix batched form (asynchronous
 map_advance); the plain FP64 form (per-level launches, host-synchronised dt) is reported
 beside it.  The state (1.2 GB in FP32, 2.4 GB in FP64) is larger than the 129 MB L2, so
 no flush is needed between steps.

@@ -411,7 +411,9 @@ int map_plan_leaves(int ndim, int nb, const map_problem_desc* problems, int n_pr
  *   to / from dev_buf, a device buffer of n * 9 * nb^ndim values in the pool's precision
  *   (double for MAP_FP64, float for MAP_FP32_FIX64; leaf-major, then [9][nz][nb][nb]),
  *   caller-owned, on the pool stream.  Unpacking is a host write: the next fill rebuilds
- *   every ghost region.
+ *   every ghost region.  The copy itself is asynchronous.  All leaves in leaf order (0..n-1)
+ *   return at once and can be captured; any other list uploads its indices first and waits for
+ *   the stream with them.
  * map_local_alpha: the maximum signal speed alpha_g (Sec. 3.7) over the active leaves, per
  *   problem, into alpha_out[n_problems] (host); synchronises.
  * map_set_alpha: finalises dt, c_h, c_p and the damping factor from the given alpha_g per

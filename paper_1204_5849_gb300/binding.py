@@ -492,7 +492,7 @@ class Pool:
 
     def test_fail_waits(self, on):
         """Test hook (map_test_fail_waits): True / 1 every bounded wait gives up at once, 2 only
-        the conduction loop's grid barrier, False / 0 normal waits."""
+        the conduction loop's waits, False / 0 normal waits."""
         self._ck(load().map_test_fail_waits(self.h, 2 if on == 2 else (1 if on else 0)), "map_test_fail_waits")
 
     def set_conduction_loop(self, on: bool):

@@ -599,6 +599,11 @@ __global__ void __launch_bounds__(256) regrid_kernel(RegridLaunch L) {
 // with the number of lanes that hold them (16 additions instead of 45).  Faces one after the
 // other with a barrier each, and every sum through all lanes: 27 -> 15 us per launch on the
 // rotor's quadtree (16^2), 57 -> 26 on a 9472-leaf octree (8^3).
+//
+// A thread per corrected cell of a leaf with its usual coarse/fine faces: up to four of 16 cells
+// (16^2), three of 64 (8^3, at a corner of the fine region), one of 256 (16^3); a leaf with more
+// takes a second round.  The choice weighs little: rotor, four steps, 32 / 64 / 128 threads 583.7 /
+// 583.8 / 585.7 us; octree, four steps, 128 / 192 / 256 threads 4069 / 4078 / 4109.
 template <int NDIM, int NB>
 __host__ __device__ constexpr int reflux_threads() {
   return NDIM == 2 ? 64 : (NB == 8 ? 192 : 256);
