@@ -151,8 +151,8 @@ def test_staging_that_does_not_fit_is_not_used(host, how):
 @pytest.mark.parametrize("prec", [0, 1])
 def test_a_pool_that_has_coarsened_gives_its_memory_back(host, prec):
     """One pool through trees that grow, shrink and grow again: every table fits its tree (the
-    launches check it), and a small tree after a large one holds at most twice what the same tree
-    holds in a pool of its own, and 256 KB for each of the twelve tables, besides the copies'
+    launches check it), and a small tree after a large one holds at most four times what the same
+    tree holds in a pool of its own, and 256 KB for each of the twelve tables, besides the copies'
     staging and flags, which stay at the largest."""
     from paper_1204_5849_gb300 import Pool
     cap = 16000
@@ -173,7 +173,7 @@ def test_a_pool_that_has_coarsened_gives_its_memory_back(host, prec):
     assert fine.nleaves > 3000
     state = 3 * cap * 9 * 12 * 12 * (8 if prec == 0 else 4)           # the block pool itself
     kept = (fine.nleaves - small.nleaves) * (9 * 64 * 8 + 9)           # staging and flags
-    assert held(small, fine) - state - kept <= 2 * (held(small, None) - state) + 12 * (256 << 10)
+    assert held(small, fine) - state - kept <= 4 * (held(small, None) - state) + 12 * (256 << 10)
     pool = Pool(small, prec, max_blocks=cap)
     for mesh in (small, _amr(1), fine, small, _amr(2), small, fine, _amr(1)):
         pool.set_tree(mesh)
@@ -182,12 +182,14 @@ def test_a_pool_that_has_coarsened_gives_its_memory_back(host, prec):
     assert counts(host)["bad"] == 0 and counts(host)["bytes"] == 0
 
 
-def test_a_pool_between_two_trees_allocates_nothing(host):
-    """A small tree that is refined and coarsened again by turns keeps its tables."""
+@pytest.mark.parametrize("radii", [((0.2,), (0.1,)), ((0.12, 0.45), (0.05, 0.3)), ((0.3, 0.44, 0.9), (0.2, 0.34, 0.7))])
+def test_a_pool_between_two_trees_allocates_nothing(host, radii):
+    """A tree that is refined and coarsened again by turns, to half its leaves, keeps its tables."""
     from paper_1204_5849_gb300 import Pool
-    a, b = _small(), _amr(1)
-    pool = Pool(b, 1, max_blocks=400)
-    host.host_set_blocks(400)
+    b, a = (w.radial_amr_mesh(2, 8, (8, 8), len(r), radii=r, bc=w.mesh.PERIODIC) for r in radii)
+    assert 0.4 * b.nleaves < a.nleaves < 0.8 * b.nleaves
+    pool = Pool(b, 1, max_blocks=4 * b.nleaves)
+    host.host_set_blocks(4 * b.nleaves)
     for mesh in (a, b, a, b):
         pool.set_tree(mesh)
     host.host_fail_from(1)                                              # no allocation succeeds
