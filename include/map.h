@@ -195,7 +195,7 @@ int map_step(map_pool* pool, const map_params* p);
  * step after the state changed outside this call.  The first steps after a change of the tree,
  * the parameters or the launch settings are plain launches on the pool's stream; later ones of
  * three launches and more are captured and replayed, four steps to a CUDA graph (the states are
- * the same either way).  The call returns early unless it enqueues more than the driver queues
+ * the same either way).  The call returns early unless it enqueues more than CUDA queues
  * for a stream, about a thousand launches or graphs: then it waits for room.  Under a capture of
  * the stream by the caller every step is plain.  map_get_speeds reads the last dt. */
 int map_advance(map_pool* pool, const map_params* p, int nsteps);

@@ -239,7 +239,7 @@ def test_schemes_that_alternate_keep_their_block_lists(host):
 
 def test_long_advances_do_not_wait_for_their_launches(host):
     """map_advance on a refined mesh: after its first steps the host enqueues four steps at a time,
-    so several hundred of them fit the driver's queue; the count of kernels is that of plain steps.
+    so several hundred of them fit CUDA's queue; the count of kernels is that of plain steps.
     A change of parameters, tree or launch settings starts anew, and a caller's capture holds plain
     launches only."""
     from paper_1204_5849_gb300 import Pool
